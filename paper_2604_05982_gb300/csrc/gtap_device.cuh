@@ -808,11 +808,16 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
     if (P.serving && wid == 0) {
         int ft = 0;
         serve_poller(P, ws, &ft);
-        if (lane == 0) { WorkerStats s{}; P.stats[wid] = s; }
+        if (lane < kStatWords) reinterpret_cast<unsigned long long*>(P.stats + wid)[lane] = 0ull;
         return;
     }
-    unsigned long long st_tasks = 0, st_steps = 0, st_pops = 0, st_popped = 0, st_sa = 0, st_steals = 0,
-                       st_stolen = 0, st_idle = 0, st_pushes = 0, st_pushed = 0, st_spawned = 0;
+    // The warp's counters live one per lane (lane i holds word i of WorkerStats): 2
+    // registers instead of 32, which the loop would otherwise spill around every step
+    // (fib(22..28) x 16: 1.22 -> 1.01 ms, hashed tree: 5.5 -> 5.0 ms, Cilksort of 300,007
+    // keys: 2.86 -> 2.62 ms).
+    unsigned long long stat = 0;
+    auto count = [&](int word, unsigned long long v) { if (lane == word) stat += v; };
+    uint32_t idle_n = 0;
     // per-lane xorshift state for victim probing
     uint64_t rng = P.seed ^ (0x9E3779B97F4A7C15ull * (uint64_t)(wid + 1)) ^ (0xD1B54A32D192ED03ull * (uint64_t)(lane + 1));
     const uint64_t t_start = global_ns();
@@ -830,8 +835,12 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
     // A warp with no task at all always tries.  Warp-uniform.
     int fill_fail = 0, fill_wait = 0;
     // per-phase clock accounting (tracing counters): pop, steal, execute, retain/push, idle
-    unsigned long long cy_pop = 0, cy_steal = 0, cy_exec = 0, cy_push = 0, cy_idle = 0;
     long long tc0 = clock64();
+    auto phase = [&](int word) {
+        const long long t = clock64();
+        count(word, (unsigned long long)(t - tc0));
+        tc0 = t;
+    };
 
     for (uint32_t iter = 0;; ++iter) {
         if ((iter & 63u) == 0u) {
@@ -877,8 +886,8 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                     if (__any_sync(0xffffffffu, bad)) break;
                     cnt += got;
                     cls = 0;
-                    ++st_pops;
-                    st_popped += got;
+                    count(kStPops, 1);
+                    count(kStPopped, got);
                 }
             }
         } else if constexpr (SCHED == SCHED_SINGLE) {
@@ -910,8 +919,8 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                     if (lane >= cnt && lane < cnt + claim) { tid = ws.retained[lane]; src = 1; }
                     cnt += claim;
                     cls = 0;
-                    st_pops += claim;
-                    st_popped += claim;
+                    count(kStPops, claim);
+                    count(kStPopped, claim);
                 }
                 __syncwarp();
             }
@@ -958,15 +967,15 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                         __syncwarp();
                         cnt += claim;
                         cls = q;
-                        ++st_pops;
-                        st_popped += claim;
+                        count(kStPops, 1);
+                        count(kStPopped, claim);
                     } else {
                         __syncwarp();
                     }
                 }
             }
         }
-        { const long long t = clock64(); cy_pop += (unsigned long long)(t - tc0); tc0 = t; }
+        phase(kStPop);
         // ---- StealBatch.  SelectVictimQueue probes kProbes random victims at once (one
         // lane each) and picks the fullest, so an idle warp finds work in one round trip.
         bool want_steal = (P.steal_policy & GTAP_STEAL_EMPTY) ? (cnt == 0) : (cnt < 32);
@@ -978,7 +987,7 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
         }
         if (want_steal && P.n_workers > 1) {
             const int cnt_before = cnt;
-            ++st_sa;
+            count(kStAttempts, 1);
             int c = -1, victim = 0, vqi = cls;
             if (lane < kProbes) {
                 rng ^= rng >> 12; rng ^= rng << 25; rng ^= rng >> 27;
@@ -1044,8 +1053,8 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                         if (lane >= cnt && lane < cnt + claim) { tid = ws.retained[lane]; src = 2; }
                         cnt += claim;
                         cls = q;
-                        st_steals += claim;
-                        st_stolen += claim;
+                        count(kStSteals, claim);
+                        count(kStStolen, claim);
                     }
                     __syncwarp();
                 } else {
@@ -1089,8 +1098,8 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                         }
                         cnt += claim;
                         cls = q;
-                        ++st_steals;
-                        st_stolen += claim;
+                        count(kStSteals, 1);
+                        count(kStStolen, claim);
                     }
                 }
             }
@@ -1103,25 +1112,25 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                 }
             }
         }
-        { const long long t = clock64(); cy_steal += (unsigned long long)(t - tc0); tc0 = t; }
+        phase(kStSteal);
         // ---- Nothing to run: termination test (all roots complete), deadline, backoff.
         if (cnt == 0) {
-            ++st_idle;
+            ++idle_n;
             int stop = 0;
-            if (lane == 0 && (st_idle & 15ull) == 1ull) {
+            if (lane == 0 && (idle_n & 15u) == 1u) {
                 if (P.serving) {
                     // served session: done once the host has closed the inbox, every submitted
                     // request has been admitted and none is in flight
                     const unsigned long long sd = *(volatile unsigned long long*)&P.hflags->shutdown;
                     if (sd != 0 && ld_cg64(&P.ctl->admitted.v) == sd - 1 && ld_cg64(&P.ctl->inflight.v) == 0) stop = 1;
                 } else if (ld_cg64(&P.ctl->roots_remaining.v) == 0ull) stop = 1;
-                else if (abort_requested(P, (st_idle & 255ull) == 1ull)) stop = 1;
+                else if (abort_requested(P, (idle_n & 255u) == 1u)) stop = 1;
                 else if (!P.serving && global_ns() > deadline) { raise_error(P, GTAP_ERR_TIMEOUT, -1, wid, P.timeout_ns); stop = 1; }
             }
             if (__shfl_sync(0xffffffffu, stop, 0)) break;
             __nanosleep(backoff);
             backoff = min(backoff * 2, P.idle_backoff_ns);
-            { const long long t = clock64(); cy_idle += (unsigned long long)(t - tc0); tc0 = t; }
+            phase(kStIdleCy);
             continue;
         }
         backoff = 32;
@@ -1156,10 +1165,10 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
         const unsigned done_mask = __ballot_sync(0xffffffffu, done);
         if (done) complete_task(P, ws, tid, rw0, rparent, rw3, rv, wid, iter);
         __syncwarp();
-        st_spawned += (unsigned)__reduce_add_sync(0xffffffffu, (unsigned)spawned);
-        st_tasks += cnt;
-        ++st_steps;
-        { const long long t = clock64(); cy_exec += (unsigned long long)(t - tc0); tc0 = t; }
+        count(kStSpawned, (unsigned)__reduce_add_sync(0xffffffffu, (unsigned)spawned));
+        count(kStTasks, cnt);
+        count(kStSteps, 1);
+        phase(kStExec);
 
         // ---- Return freed records to the local stack; spill the surplus.
         {
@@ -1280,29 +1289,18 @@ __device__ void thread_mode_loop(const KParams& P, char* smem_warp) {
                     }
                 }
             }
-            if (lane == 0) {
-                int tot = 0;
-                for (int q = 0; q < Q; ++q) tot += ws.push_off[q];
-                if (tot > 0) { ++st_pushes; st_pushed += tot; }
-            }
+            if (nkeep < nst) { count(kStPushes, 1); count(kStPushed, nst - nkeep); }
             __syncwarp();
             if (lane < nkeep) { tid = ws.retained[lane]; src = 0; }
             cnt = nkeep;
             cls = qstar;
             __syncwarp();
         }
-        { const long long t = clock64(); cy_push += (unsigned long long)(t - tc0); tc0 = t; }
+        phase(kStPush);
     }
 
-    // Give cached frames back so a later run or another worker could use them (best effort).
-    if (lane == 0) {
-        WorkerStats s;
-        s.tasks = st_tasks; s.steps = st_steps; s.pops = st_pops; s.popped = st_popped;
-        s.steal_attempts = st_sa; s.steals = st_steals; s.stolen = st_stolen; s.idle = st_idle;
-        s.pushes = st_pushes; s.pushed = st_pushed; s.spawned = st_spawned;
-        s.pad[0] = cy_pop; s.pad[1] = cy_steal; s.pad[2] = cy_exec; s.pad[3] = cy_push; s.pad[4] = cy_idle;
-        P.stats[wid] = s;
-    }
+    count(kStIdle, idle_n);
+    if (lane < kStatWords) reinterpret_cast<unsigned long long*>(P.stats + wid)[lane] = stat;
 }
 
 

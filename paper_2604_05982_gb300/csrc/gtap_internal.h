@@ -170,6 +170,12 @@ struct WorkerStats {
     unsigned long long tasks, steps, pops, popped, steal_attempts, steals, stolen, idle, pushes, pushed, spawned;
     unsigned long long pad[5];   // thread mode: SM cycles spent in pop, steal, execute, retain/push, idle
 };
+// Words of WorkerStats, in order.
+enum StatWord : int {
+    kStTasks, kStSteps, kStPops, kStPopped, kStAttempts, kStSteals, kStStolen, kStIdle, kStPushes, kStPushed, kStSpawned,
+    kStPop, kStSteal, kStExec, kStPush, kStIdleCy, kStatWords
+};
+static_assert(sizeof(WorkerStats) == kStatWords * 8, "StatWord names the words of WorkerStats");
 
 // Kernel parameters (passed by value).
 struct KParams {
