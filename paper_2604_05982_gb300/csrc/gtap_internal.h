@@ -232,7 +232,8 @@ enum DebugFault : unsigned long long {
     DBG_DOUBLE_ALLOC = 1, DBG_DOUBLE_FREE = 2, DBG_EXEC_NOT_ALLOCATED = 3, DBG_BAD_ID = 4,
 };
 
-// Shared-memory sizing (thread mode: per warp; block mode: per block, runtime part).
+// Shared-memory sizing (thread mode: per warp after a small per-block part; block mode: per block, runtime part).
+constexpr int kThreadBlockSmem = 16;   // BlockIdle
 GTAP_HD constexpr int thread_fcap(int maxspawn) { return 32 * maxspawn + 3 * kChunk + 32; }
 GTAP_HD constexpr int thread_scap(int maxspawn) { return 32 * (maxspawn > 1 ? maxspawn : 1); }
 GTAP_HD constexpr int thread_warp_smem(int maxspawn) {

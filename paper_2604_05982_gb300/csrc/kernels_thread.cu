@@ -66,8 +66,11 @@ constexpr int thread_min_blocks() {
 template <unsigned PSET, int SCHED>
 __global__ void __launch_bounds__(256, thread_min_blocks<PSET>()) thread_kernel(KParams P) {
     extern __shared__ __align__(16) char smem[];
+    BlockIdle* bidle = reinterpret_cast<BlockIdle*>(smem);
+    if (threadIdx.x == 0) { bidle->token = 0; bidle->stop = 0; }
+    __syncthreads();
     const int wib = threadIdx.x >> 5;
-    thread_mode_loop<ThreadDispatch<PSET>, SCHED>(P, smem + (size_t)wib * P.warp_smem);
+    thread_mode_loop<ThreadDispatch<PSET>, SCHED>(P, bidle, smem + kThreadBlockSmem + (size_t)wib * P.warp_smem);
 }
 
 // Default scheduler for every program set; the Sec. 6.5 comparison variants for
