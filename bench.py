@@ -433,7 +433,7 @@ FP64_NOMINAL_TFLOPS = 1.25  # GB300 FP64, nominal
 
 
 def m2l_flops_per_pair(p: int) -> int:
-    """Arithmetic of one M2L translation as the kernel performs it: the Taylor
+    """Arithmetic of one M2L translation over all (p+1)(p+2)(p+3)/6 coefficients: the Taylor
     recurrence (3 flops per first-order term, 2 per second-order term, 1 for the
     final scaling, plus r^2, 1/r^2 and 1/r) and one FMA per (alpha, beta) term."""
     fl = 7
@@ -444,6 +444,27 @@ def m2l_flops_per_pair(p: int) -> int:
                 fl += 3 * sum(1 for x in n if x > 0) + 2 * sum(1 for x in n if x > 1) + 1
     terms = sum(1 for k1 in range(p + 1) for _ in range((k1 + 1) * (k1 + 2) // 2)
                 for k2 in range(p - k1 + 1) for _ in range((k2 + 1) * (k2 + 2) // 2))
+    return fl + 2 * terms
+
+
+def m2l_flops_per_pair_harmonic(p: int) -> int:
+    """Arithmetic of one M2L translation as the kernel performs it, over the (p+1)^2
+    coefficients with z-index 0 and 1: per order 4 factors, per coefficient a multiply-add for
+    each first- and second-order term (a multiply for the first of each) and 1 or 3 flops to
+    combine them, 2 flops per z = 2 entry, one FMA per (alpha, beta) term."""
+    fl = 7 + 2 * p
+    terms = 0
+    for k in range(1, p + 1):
+        fl += 2
+        for c in (0, 1):
+            for b in range(k - c + 1):
+                n = (k - b - c, b)
+                first, second = sum(1 for x in (*n, c) if x > 0), sum(1 for x in n if x > 1)
+                fl += 2 * first - 1 + (2 * second - 1 + 3 if second else 1)
+        fl += 2 * (k - 1)
+    for k1 in range(p + 1):
+        for k2 in range(p - k1 + 1):
+            terms += (2 * k1 + 1) * (2 * k2 + 1)
     return fl + 2 * terms
 
 
@@ -550,7 +571,7 @@ def run_fmm(args):
     breakdown = {dist: {k: med(dist, k) for k in keys} for dist in sets}
     info = {dist: phases[dist][-1] for dist in sets}
     # roofline of the dominant kernel (M2L): ALU bound, peak from unit counts and the maximum clock
-    fl = m2l_flops_per_pair(FMM_P)
+    fl = m2l_flops_per_pair_harmonic(FMM_P)
     pairs = sum(info[dd]["n_m2l"] for dd in sets)
     m2l_ms = sum(breakdown[dd]["ms_m2l"] for dd in sets)
     achieved = pairs * fl / (m2l_ms / 1e3) / 1e12

@@ -15,6 +15,7 @@
 // top levels stay in double.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "fmm_internal.h"
@@ -275,65 +276,189 @@ __global__ void k_m2l(EvalBufs e) {
     }
 }
 
-// M2L in FP32 with the whole expansion in registers, one warp per target
-// cell and one source cell per lane.  In the scaled variables
+// M2L with the expansion in registers, one warp per target cell and one source
+// cell per lane.  In the scaled variables
 //   Tt_n = n! T_n,   Mt_a = (-1)^|a| M_a / a!,   Lt_b = b! L_b
-// the translation is a plain correlation, Lt_b = sum_a Tt_{a+b} Mt_a, one FMA
-// per term, and the recurrence for Tt has compile-time coefficients:
-//   |n| r^2 Tt_n = -(2|n|-1) sum_i n_i x_i Tt_{n-e_i} - (|n|-1) sum_i n_i (n_i-1) Tt_{n-2e_i}.
+// the translation is a plain correlation, Lt_b = sum_a Tt_{a+b} Mt_a.
+//
+// 1/r is harmonic: Tt_{n+2ex} + Tt_{n+2ey} + Tt_{n+2ez} = 0.  So every index
+// with z >= 2 folds onto indices with z in {0, 1},
+//   Tt_{(x, y, z)} = (-1)^m sum_j C(m, j) Tt_{(x+2j, y+2(m-j), z-2m)},  m = z / 2,
+// the multipole is folded once per cell (k_fold_m), Lt is accumulated for z in
+// {0, 1} only (its truncated sum is harmonic as well) and unfolded once per
+// target.  (p+1)^2 coefficients instead of (p+1)(p+2)(p+3)/6: at p = 6, 49
+// instead of 84, 532 multiply-adds a pair instead of 924, and a recurrence over
+// 49 coefficients (plus 15 sums for z = 2) instead of 84.
 // The order P is a template parameter so that every index is a constant and
 // the compiler keeps Tt and Lt in registers.
 __host__ __device__ constexpr int cidx(int a, int b, int c) {
     return (a + b + c) * (a + b + c + 1) * (a + b + c + 2) / 6 + (b + c) * (b + c + 1) / 2 + c;
 }
-__host__ __device__ constexpr int row_stride(int p) { return (n_coef(p) + 3) / 4 * 4; }
+// coefficients with z in {0, 1}: order k starts at k^2, its z = 0 entries by y, then z = 1 by y
+__host__ __device__ constexpr int n_harm(int p) { return (p + 1) * (p + 1); }
+__host__ __device__ constexpr int hidx(int a, int b, int c) {
+    return (a + b + c) * (a + b + c) + (c ? (a + b + c) + 1 + b : b);
+}
+// z = 2 entries of the derivative table, after the n_harm(p) others
+__host__ __device__ constexpr int n_harm2(int p) { return p * (p - 1) / 2; }
+__host__ __device__ constexpr int tidx(int p, int a, int b, int c) {
+    return c < 2 ? hidx(a, b, c) : n_harm(p) + (a + b + 1) * (a + b) / 2 + b;
+}
+__host__ __device__ constexpr int row_stride(int p) { return (n_harm(p) + 3) / 4 * 4; }
 
-template <int P>
-__device__ __forceinline__ void taylor_scaled(float x, float y, float z, float* T) {
-    const float r2 = x * x + y * y + z * z;
-    const float ir = rsqrtf(r2);
-    const float ir2 = ir * ir;
+// Row `cell` of Ms: the folded multipole sum_{m, j} (-1)^m C(m, j) Mt, in FP64,
+// rounded once to the row's type; the factors (-1)^|a| / a! come from a
+// per-coefficient table (an FP64 divide is a long sequence on the FP64 pipe,
+// the narrowest pipe of this GPU).  Row n_cells is zero: the source of idle lanes.
+template <int P, class R>
+__global__ void k_fold_m(const double* __restrict__ M, int n_cells, const double* __restrict__ mscale,
+                         R* __restrict__ Ms) {
+    constexpr int N = n_coef(P), H = n_harm(P), S = row_stride(P);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)(n_cells + 1) * S;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int cell = (int)(i / S), h = (int)(i - (long long)cell * S);
+        double v = 0.0;
+        if (h < H && cell < n_cells) {
+            int k = 0;
+            while ((k + 1) * (k + 1) <= h) ++k;
+            const int r = h - k * k, c = r > k ? 1 : 0, b = c ? r - k - 1 : r, a = k - b - c;
+            const double* Mc = M + (size_t)cell * N;
+            for (int m = 0; 2 * m <= a + b; ++m) {
+                double binom = 1.0;   // C(m, j)
+                for (int j = 0; j <= m; ++j) {
+                    const int ax = a - 2 * j, bx = b - 2 * (m - j);
+                    if (ax >= 0 && bx >= 0) {
+                        const int id = cidx(ax, bx, c + 2 * m);
+                        const double t = binom * (Mc[id] * __ldg(mscale + id));
+                        v += (m & 1) ? -t : t;
+                    }
+                    binom = binom * (double)(m - j) / (double)(j + 1);
+                }
+            }
+        }
+        Ms[i] = (R)v;
+    }
+}
+
+// Tt_n of the displacement (x, y, z) for z-index 0, 1 and 2, by
+//   |n| r^2 Tt_n = -(2|n|-1) sum_i n_i x_i Tt_{n-e_i} - (|n|-1) sum_i n_i (n_i-1) Tt_{n-2e_i}.
+// T[i * LD] is coefficient i (LD = 32: a lane's column of a shared table).
+template <int P, int LD, class R>
+__device__ __forceinline__ void taylor_harmonic(R x, R y, R z, R ir, R ir2, R* T) {
+    R ax[P + 1], by[P + 1];
+#pragma unroll
+    for (int k = 1; k <= P; ++k) { ax[k] = (R)k * x; by[k] = (R)k * y; }
     T[0] = ir;
 #pragma unroll
     for (int k = 1; k <= P; ++k) {
-        const float ck = -(2.f * k - 1.f) / (float)k, dk = -((float)k - 1.f) / (float)k;
+        const R ck = (R)(-(2.0 * k - 1.0) / (double)k) * ir2, dk = (R)(-((double)k - 1.0) / (double)k) * ir2;
 #pragma unroll
-        for (int a = k; a >= 0; --a) {
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
-            for (int b = k - a; b >= 0; --b) {
-                const int c = k - a - b;
-                float acc = 0.f;
-                if (a > 0) acc += (ck * a) * x * T[cidx(a - 1, b, c)];
-                if (b > 0) acc += (ck * b) * y * T[cidx(a, b - 1, c)];
-                if (c > 0) acc += (ck * c) * z * T[cidx(a, b, c - 1)];
-                if (a > 1) acc += (dk * a * (a - 1)) * T[cidx(a - 2, b, c)];
-                if (b > 1) acc += (dk * b * (b - 1)) * T[cidx(a, b - 2, c)];
-                if (c > 1) acc += (dk * c * (c - 1)) * T[cidx(a, b, c - 2)];
-                T[cidx(a, b, c)] = acc * ir2;
+            for (int b = 0; b <= k - c; ++b) {
+                const int a = k - b - c;
+                R s1 = 0, s2 = 0;
+                if (a > 0) s1 += ax[a] * T[LD * hidx(a - 1, b, c)];
+                if (b > 0) s1 += by[b] * T[LD * hidx(a, b - 1, c)];
+                if (c > 0) s1 += z * T[LD * hidx(a, b, c - 1)];
+                if (a > 1) s2 += (R)(a * (a - 1)) * T[LD * hidx(a - 2, b, c)];
+                if (b > 1) s2 += (R)(b * (b - 1)) * T[LD * hidx(a, b - 2, c)];
+                T[LD * hidx(a, b, c)] = (a > 1 || b > 1) ? ck * s1 + dk * s2 : ck * s1;
             }
+    }
+#pragma unroll
+    for (int k = 2; k <= P; ++k)
+#pragma unroll
+        for (int b = 0; b <= k - 2; ++b)
+            T[LD * tidx(P, k - 2 - b, b, 2)] = -(T[LD * hidx(k - b, b, 0)] + T[LD * hidx(k - 2 - b, b + 2, 0)]);
+}
+
+// L_b += sum_a Tt_{a+b} row_a over one source row (V: the vector type of its loads).
+template <int P, int LD, class R, class V>
+__device__ __forceinline__ void m2l_accumulate(const R* T, const R* __restrict__ row, R* L) {
+    constexpr int W = (int)(sizeof(V) / sizeof(R));
+    R mv[W];
+#pragma unroll
+    for (int k1 = 0; k1 <= P; ++k1)
+#pragma unroll
+        for (int c1 = 0; c1 < 2; ++c1)
+#pragma unroll
+            for (int b1 = 0; b1 <= k1 - c1; ++b1) {
+                const int a1 = k1 - b1 - c1, ia = hidx(a1, b1, c1);
+                if (ia % W == 0) {
+                    const V v = __ldg(reinterpret_cast<const V*>(row) + ia / W);
+                    memcpy(mv, &v, sizeof(V));
+                }
+                const R m = mv[ia % W];
+#pragma unroll
+                for (int k2 = 0; k2 <= P - k1; ++k2)
+#pragma unroll
+                    for (int c2 = 0; c2 < 2; ++c2)
+#pragma unroll
+                        for (int b2 = 0; b2 <= k2 - c2; ++b2) {
+                            const int a2 = k2 - b2 - c2;
+                            R& l = L[hidx(a2, b2, c2)];
+                            l += T[LD * tidx(P, a1 + a2, b1 + b2, c1 + c2)] * m;
+                        }
+            }
+}
+
+// One round of a butterfly reduction that halves the vector: the lane keeps the
+// half its bit O selects and gives the other to its partner.
+template <int O, int N, class R>
+__device__ __forceinline__ void butterfly_halve(R* v, int* base) {
+    const bool up = (threadIdx.x & O) != 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const R mine = up ? v[i + N] : v[i], give = up ? v[i] : v[i + N];
+        v[i] = mine + __shfl_xor_sync(0xffffffffu, give, O);
+    }
+    if (up) *base += N;
+}
+
+// Sum the 32 lanes' partial expansions: a butterfly that halves the vector each
+// round leaves every lane with PAD / 32 finished sums (62 shuffles at p = 6; one
+// full reduction per coefficient would take 245), which go to `out` (shared, PAD
+// entries).  Then the warp unfolds and writes L_b = Lt_b / b! in FP64.
+template <int P, class R>
+__device__ __forceinline__ void m2l_finish(R (&L)[n_harm(P)], R* out, const EvalBufs& e, int tgt) {
+    constexpr int N = n_coef(P), H = n_harm(P), PAD = (H + 31) / 32 * 32;
+    const int lane = threadIdx.x & 31;
+    R v[PAD];
+#pragma unroll
+    for (int i = 0; i < PAD; ++i) v[i] = i < H ? L[i] : (R)0;
+    int base = 0;
+    butterfly_halve<16, PAD / 2>(v, &base);
+    butterfly_halve<8, PAD / 4>(v, &base);
+    butterfly_halve<4, PAD / 8>(v, &base);
+    butterfly_halve<2, PAD / 16>(v, &base);
+    butterfly_halve<1, PAD / 32>(v, &base);
+#pragma unroll
+    for (int i = 0; i < PAD / 32; ++i) out[base + i] = v[i];
+    __syncwarp();
+    for (int i = lane; i < N; i += 32) {
+        const short3 n = e.tab.mi[i];
+        const int m = n.z >> 1, c = n.z & 1;
+        double s = 0.0, binom = (m & 1) ? -1.0 : 1.0;   // (-1)^m C(m, j)
+        for (int j = 0; j <= m; ++j) {
+            s += binom * (double)out[hidx(n.x + 2 * j, n.y + 2 * (m - j), c)];
+            binom = (m == 3) ? (j == 0 || j == 1 ? -3.0 : -1.0) : (m == 2) ? (j == 0 ? 2.0 : 1.0) : binom;
         }
+        e.L[(size_t)tgt * N + i] = s * __ldg(e.tab.lscale + i);
     }
 }
 
-// Ms[cell][row_stride(P)] = (-1)^|a| M_a / a! in FP32; the factors come from a
-// per-coefficient table (an FP64 divide is a long sequence on the FP64 pipe,
-// the narrowest pipe of this GPU).
-template <int P>
-__global__ void k_scale_m(const double* __restrict__ M, int n_cells, const double* __restrict__ mscale,
-                          float* __restrict__ Ms) {
-    constexpr int N = n_coef(P), S = row_stride(P);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)n_cells * S;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i / S), j = (int)(i - (long long)c * S);
-        Ms[i] = (j < N) ? (float)(M[(size_t)c * N + j] * __ldg(mscale + j)) : 0.f;
-    }
-}
+constexpr int kM2lWarps = 4;
 
-// 3 resident blocks per SM (at most 168 registers, a few spills) measured 5 % faster than
-// the unconstrained 229 registers at 2 blocks, and than 4 blocks with heavy spilling.
+// Bound by FP32 issue and by the lanes' uncoalesced row reads (208 B a source).
+// 49 + 64 expansion and derivative registers fit 128, so 4 blocks (16 warps)
+// stay resident; over 84 coefficients it took 168 registers at 3 blocks.
+// N = 2^20 uniform, p = 6: 2.29 -> 1.70 ms (fold included); Plummer 3.88 -> 2.86 ms.
+// Error against the FP64 form there: 9.2e-7 -> 7.6e-7 and 1.4e-6 -> 1.1e-6.
 template <int P>
-__global__ void __launch_bounds__(128, 3) k_m2l_reg(EvalBufs e, const float* __restrict__ Ms) {
-    constexpr int N = n_coef(P), S = row_stride(P);
+__global__ void __launch_bounds__(32 * kM2lWarps, 4) k_m2l_reg(EvalBufs e, const float* __restrict__ Ms) {
+    constexpr int H = n_harm(P), S = row_stride(P);
+    __shared__ float sums[kM2lWarps][(H + 31) / 32 * 32];
     const int lane = threadIdx.x & 31;
     const int tgt = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     if (tgt >= e.n_cells) return;
@@ -342,161 +467,53 @@ __global__ void __launch_bounds__(128, 3) k_m2l_reg(EvalBufs e, const float* __r
     // exact integer displacement on the level-21 lattice, one FP32 scaling
     const int4 lt = e.lat[tgt];
     const float u = e.lat_unit;
-    float L[N];
+    const int far = e.m2l_src[s0];   // an idle lane's displacement: any valid one, times the zero row
+    float L[H];
 #pragma unroll
-    for (int i = 0; i < N; ++i) L[i] = 0.f;
+    for (int i = 0; i < H; ++i) L[i] = 0.f;
     for (int base = s0; base < s1; base += 32) {
         const int s = base + lane;
-        const bool valid = s < s1;
-        const int src = valid ? e.m2l_src[s] : e.m2l_src[s0];
+        const int src = s < s1 ? e.m2l_src[s] : far;
         const int4 ls = __ldg(e.lat + src);
         const float x = (float)(lt.x - ls.x) * u, y = (float)(lt.y - ls.y) * u, z = (float)(lt.z - ls.z) * u;
-        float T[N];
-        taylor_scaled<P>(x, y, z, T);
-        const float wgt = valid ? 1.f : 0.f;
-        const float4* row = reinterpret_cast<const float4*>(Ms + (size_t)src * S);
-        float4 mv = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int k1 = 0; k1 <= P; ++k1)
-#pragma unroll
-            for (int a1 = k1; a1 >= 0; --a1)
-#pragma unroll
-                for (int b1 = k1 - a1; b1 >= 0; --b1) {
-                    const int c1 = k1 - a1 - b1;
-                    const int ia = cidx(a1, b1, c1);
-                    if ((ia & 3) == 0) mv = __ldg(row + ia / 4);
-                    const float m = wgt * ((ia & 3) == 0 ? mv.x : (ia & 3) == 1 ? mv.y : (ia & 3) == 2 ? mv.z : mv.w);
-#pragma unroll
-                    for (int k2 = 0; k2 <= P - k1; ++k2)
-#pragma unroll
-                        for (int a2 = k2; a2 >= 0; --a2)
-#pragma unroll
-                            for (int b2 = k2 - a2; b2 >= 0; --b2) {
-                                const int c2 = k2 - a2 - b2;
-                                L[cidx(a2, b2, c2)] = fmaf(T[cidx(a1 + a2, b1 + b2, c1 + c2)], m, L[cidx(a2, b2, c2)]);
-                            }
-                }
+        const float ir = rsqrtf(x * x + y * y + z * z);
+        float T[H + n_harm2(P) + 1];
+        taylor_harmonic<P, 1>(x, y, z, ir, ir * ir, T);
+        m2l_accumulate<P, 1, float, float4>(T, Ms + (size_t)(s < s1 ? src : e.n_cells) * S, L);
     }
-    // sum the lanes' partial expansions, then lane l writes L_b = Lt_b / b! for
-    // b = l, l + 32, l + 64 (selected by register moves; one FP64 multiply each)
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        float v = L[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        L[i] = v;
-    }
-    constexpr int R = (N + 31) / 32;
-    float w[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = 0.f;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-        if ((i & 31) == lane) w[i >> 5] = L[i];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (lane + 32 * r < N) e.L[(size_t)tgt * N + lane + 32 * r] = (double)w[r] * __ldg(e.tab.lscale + lane + 32 * r);
+    m2l_finish<P>(L, sums[threadIdx.x >> 5], e, tgt);
 }
 
-// FP64 M2L in the same scaled form: the local expansion stays in registers,
-// the Taylor coefficients of each lane's source go to the lane's column of a
-// shared-memory table (FP64 registers cannot hold both).  The FP64 pipe, not
-// the shared-memory bandwidth, bounds this kernel.
+// FP64: the local expansion stays in registers, the Taylor coefficients of each
+// lane's source go to the lane's column of a shared-memory table.  The FP64
+// pipe, not the shared-memory bandwidth, bounds this kernel (N = 2^20 uniform:
+// 87.0 -> 49.1 ms, Plummer 151 -> 85.8 ms with the harmonic form).
 template <int P>
-__global__ void k_scale_m64(const double* __restrict__ M, int n_cells, const double* __restrict__ mscale,
-                            double* __restrict__ Ms) {
-    constexpr int N = n_coef(P), S = row_stride(P);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < (long long)n_cells * S;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i / S), j = (int)(i - (long long)c * S);
-        Ms[i] = (j < N) ? M[(size_t)c * N + j] * __ldg(mscale + j) : 0.0;
-    }
-}
-
-constexpr int kM2l64Warps = 4;
-
-template <int P>
-__global__ void __launch_bounds__(32 * kM2l64Warps) k_m2l_reg64(EvalBufs e, const double* __restrict__ Ms) {
-    constexpr int N = n_coef(P), S = row_stride(P);
+__global__ void __launch_bounds__(32 * kM2lWarps) k_m2l_reg64(EvalBufs e, const double* __restrict__ Ms) {
+    constexpr int H = n_harm(P), S = row_stride(P), NT = H + n_harm2(P);
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    double* T = reinterpret_cast<double*>(sm_raw) + (size_t)wib * N * 32 + lane;   // T[i * 32]
+    double* T = reinterpret_cast<double*>(sm_raw) + (size_t)wib * NT * 32 + lane;   // T[i * 32]
     const int tgt = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     if (tgt >= e.n_cells) return;
     const int s0 = e.m2l_off[tgt], s1 = e.m2l_off[tgt + 1];
     if (s0 == s1) return;
     const Dbl4 g = e.geom[tgt];
-    double L[N];
+    const int far = e.m2l_src[s0];
+    double L[H];
 #pragma unroll
-    for (int i = 0; i < N; ++i) L[i] = 0.0;
+    for (int i = 0; i < H; ++i) L[i] = 0.0;
     for (int base = s0; base < s1; base += 32) {
         const int s = base + lane;
-        const bool valid = s < s1;
-        const int src = valid ? e.m2l_src[s] : e.m2l_src[s0];
+        const int src = s < s1 ? e.m2l_src[s] : far;
         const Dbl4 gs = e.geom[src];
         const double x = __dsub_rn(g.x, gs.x), y = __dsub_rn(g.y, gs.y), z = __dsub_rn(g.z, gs.z);
         const double r2 = x * x + y * y + z * z;
-        const double ir2 = 1.0 / r2;
-        T[0] = rsqrt(r2);
-#pragma unroll
-        for (int k = 1; k <= P; ++k) {
-            const double ck = -(2.0 * k - 1.0) / (double)k, dk = -((double)k - 1.0) / (double)k;
-#pragma unroll
-            for (int a = k; a >= 0; --a)
-#pragma unroll
-                for (int b = k - a; b >= 0; --b) {
-                    const int c = k - a - b;
-                    double acc = 0.0;
-                    if (a > 0) acc += (ck * a) * x * T[32 * cidx(a - 1, b, c)];
-                    if (b > 0) acc += (ck * b) * y * T[32 * cidx(a, b - 1, c)];
-                    if (c > 0) acc += (ck * c) * z * T[32 * cidx(a, b, c - 1)];
-                    if (a > 1) acc += (dk * a * (a - 1)) * T[32 * cidx(a - 2, b, c)];
-                    if (b > 1) acc += (dk * b * (b - 1)) * T[32 * cidx(a, b - 2, c)];
-                    if (c > 1) acc += (dk * c * (c - 1)) * T[32 * cidx(a, b, c - 2)];
-                    T[32 * cidx(a, b, c)] = acc * ir2;
-                }
-        }
-        const double wgt = valid ? 1.0 : 0.0;
-        const double2* row = reinterpret_cast<const double2*>(Ms + (size_t)src * S);
-        double2 mv = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int k1 = 0; k1 <= P; ++k1)
-#pragma unroll
-            for (int a1 = k1; a1 >= 0; --a1)
-#pragma unroll
-                for (int b1 = k1 - a1; b1 >= 0; --b1) {
-                    const int c1 = k1 - a1 - b1;
-                    const int ia = cidx(a1, b1, c1);
-                    if ((ia & 1) == 0) mv = __ldg(row + ia / 2);
-                    const double m = wgt * ((ia & 1) == 0 ? mv.x : mv.y);
-#pragma unroll
-                    for (int k2 = 0; k2 <= P - k1; ++k2)
-#pragma unroll
-                        for (int a2 = k2; a2 >= 0; --a2)
-#pragma unroll
-                            for (int b2 = k2 - a2; b2 >= 0; --b2) {
-                                const int c2 = k2 - a2 - b2;
-                                L[cidx(a2, b2, c2)] = fma(T[32 * cidx(a1 + a2, b1 + b2, c1 + c2)], m, L[cidx(a2, b2, c2)]);
-                            }
-                }
+        taylor_harmonic<P, 32>(x, y, z, rsqrt(r2), 1.0 / r2, T);
+        m2l_accumulate<P, 32, double, double2>(T, Ms + (size_t)(s < s1 ? src : e.n_cells) * S, L);
     }
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        double v = L[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        L[i] = v;
-    }
-    constexpr int R = (N + 31) / 32;
-    double w[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = 0.0;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-        if ((i & 31) == lane) w[i >> 5] = L[i];
-#pragma unroll
-    for (int r = 0; r < R; ++r)
-        if (lane + 32 * r < N) e.L[(size_t)tgt * N + lane + 32 * r] = w[r] * __ldg(e.tab.lscale + lane + 32 * r);
+    __syncwarp();   // the warp's table becomes the buffer of the lane sums
+    m2l_finish<P>(L, T - lane, e, tgt);
 }
 
 // L2L from the parents of one level into their children: one block per parent.
@@ -872,24 +889,24 @@ cudaError_t launch_upward(const EvalBufs& e, bool mixed, int fp64_levels, cudaSt
 
 template <int P>
 cudaError_t launch_m2l_reg(const EvalBufs& e, float* ms, cudaStream_t s) {
-    k_scale_m<P><<<grid_for((long long)e.n_cells * row_stride(P), 256, 4096), 256, 0, s>>>(e.M, e.n_cells, e.tab.mscale, ms);
-    k_m2l_reg<P><<<grid_for((long long)e.n_cells * 32, 128, 1 << 30), 128, 0, s>>>(e, ms);
+    k_fold_m<P, float><<<grid_for((e.n_cells + 1ll) * row_stride(P), 256, 4096), 256, 0, s>>>(e.M, e.n_cells, e.tab.mscale, ms);
+    k_m2l_reg<P><<<grid_for((long long)e.n_cells * 32, 32 * kM2lWarps, 1 << 30), 32 * kM2lWarps, 0, s>>>(e, ms);
     return cudaGetLastError();
 }
 
 template <int P>
 cudaError_t launch_m2l_reg64(const EvalBufs& e, double* ms, cudaStream_t s) {
-    k_scale_m64<P><<<grid_for((long long)e.n_cells * row_stride(P), 256, 4096), 256, 0, s>>>(e.M, e.n_cells, e.tab.mscale, ms);
-    const size_t sm = sizeof(double) * n_coef(P) * 32 * kM2l64Warps;
+    k_fold_m<P, double><<<grid_for((e.n_cells + 1ll) * row_stride(P), 256, 4096), 256, 0, s>>>(e.M, e.n_cells, e.tab.mscale, ms);
+    const size_t sm = sizeof(double) * std::max(n_harm(P) + n_harm2(P), (n_harm(P) + 31) / 32) * 32 * kM2lWarps;
     cudaError_t err = set_smem(k_m2l_reg64<P>, sm);
     if (err != cudaSuccess) return err;
-    k_m2l_reg64<P><<<grid_for((long long)e.n_cells * 32, 32 * kM2l64Warps, 1 << 30), 32 * kM2l64Warps, sm, s>>>(e, ms);
+    k_m2l_reg64<P><<<grid_for((long long)e.n_cells * 32, 32 * kM2lWarps, 1 << 30), 32 * kM2lWarps, sm, s>>>(e, ms);
     return cudaGetLastError();
 }
 
-// Scratch for the scaled multipoles: FP32 rows (mixed) or FP64 rows, in bytes.
+// Scratch for the folded multipoles: FP32 rows (mixed) or FP64 rows, one per cell and a zero row, in bytes.
 size_t m2l_scratch_bytes(int p, int n_cells, bool mixed) {
-    return (size_t)n_cells * row_stride(p) * (mixed ? sizeof(float) : sizeof(double));
+    return ((size_t)n_cells + 1) * row_stride(p) * (mixed ? sizeof(float) : sizeof(double));
 }
 
 cudaError_t launch_m2l(const EvalBufs& e, bool mixed, cudaStream_t s) {
