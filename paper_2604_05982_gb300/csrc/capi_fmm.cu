@@ -148,6 +148,7 @@ struct gtap_fmm {
     gtap_fmm_config cfg{};
     int p = 6, nt = 84;
     bool mixed = false;
+    int sms = 0;
     cudaStream_t s = nullptr;
     HostTables ht;
     Tables tab{};
@@ -160,7 +161,7 @@ struct gtap_fmm {
     int cell_cap = 0;
     const uint32_t* order = nullptr;
     // expansions and lists
-    DBuf M, L, m2l, p2p, counters, gcnt, gcur, m2l_off, m2l_src, p2p_off, p2p_src, ms, aux;
+    DBuf M, L, m2l, p2p, counters, gcnt, gcur, m2l_off, m2l_src, p2p_off, p2p_src, p2p_runs, ms, aux;
     long long m2l_cap = 0, p2p_cap = 0;
 
     long long n = 0;
@@ -174,7 +175,7 @@ struct gtap_fmm {
     ~gtap_fmm() {
         DBuf* all[] = {&tab_dev, &keys0, &keys1, &vals0, &vals1, &pts, &ploc, &hist, &hist_scan, &tile_sums, &box,
                        &bbox_part, &geom, &info, &lat, &lstart, &lvl_n, &lvl_total, &cnt, &off, &bounds, &flags, &M, &L,
-                       &m2l, &p2p, &counters, &gcnt, &gcur, &m2l_off, &m2l_src, &p2p_off, &p2p_src, &ms, &aux};
+                       &m2l, &p2p, &counters, &gcnt, &gcur, &m2l_off, &m2l_src, &p2p_off, &p2p_src, &p2p_runs, &ms, &aux};
         for (DBuf* b : all) b->release();
         for (cudaEvent_t& e : ev)
             if (e) cudaEventDestroy(e);
@@ -274,6 +275,13 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
     f->p = c.order;
     f->mixed = c.precision == GTAP_FMM_MIXED;
     f->s = static_cast<cudaStream_t>(c.stream);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        delete f;
+        return GTAP_ERR_CUDA;
+    }
     f->ht.build(c.order);
     f->nt = f->ht.nt;
     const HostTables& h = f->ht;
@@ -488,6 +496,7 @@ gtap_status gtap_fmm_evaluate(gtap_fmm* f, double* phi) {
         !f->m2l_src.ensure(sizeof(int) * (size_t)std::max(f->n_m2l, 1ll)) ||
         !f->p2p_src.ensure(sizeof(int) * (size_t)std::max(f->n_p2p, 1ll)) ||
         !f->tile_sums.ensure(sizeof(int) * (size_t)scan::tiles_for((long long)nc)) ||
+        !f->p2p_runs.ensure(p2p_scratch_bytes(f->mixed, f->n, f->n_p2p, f->n_leaves, f->sms)) ||
         !f->ms.ensure(m2l_scratch_bytes(f->p, f->n_cells, f->mixed)))
         return GTAP_ERR_NO_MEMORY;
     cudaEventRecord(f->ev[3], f->s);
@@ -503,7 +512,7 @@ gtap_status gtap_fmm_evaluate(gtap_fmm* f, double* phi) {
     cudaEventRecord(f->ev[5], f->s);
     if (launch_downward(e, f->mixed, f->cfg.fp64_levels, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
     cudaEventRecord(f->ev[6], f->s);
-    if (launch_leaf_eval(e, f->mixed, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
+    if (launch_leaf_eval(e, f->mixed, f->n_p2p, f->n_leaves, f->sms, f->p2p_runs.p, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
     cudaEventRecord(f->ev[7], f->s);
     if (cudaStreamSynchronize(f->s) != cudaSuccess) return GTAP_ERR_CUDA;
     f->info_h.ms_group = elapsed(f->ev[3], f->ev[4]);

@@ -1,13 +1,13 @@
 // Data-parallel FMM kernels around the traversal (Sec. 6.4.1): upward pass
 // (P2M at leaves, M2M level by level), M2L over the interaction list grouped
-// by target cell, downward pass (L2L level by level) and the leaf kernel
-// (L2P + P2P over the near-field list).  Cartesian Taylor expansions of total
+// by target cell, and downward pass (L2L level by level); the leaf kernels
+// (L2P and P2P) are in fmm_leaf.cu.  Cartesian Taylor expansions of total
 // order p about the cell centres:
 //   P2M  M_a  = sum_j q_j (x_j - c)^a
 //   M2M  M_a(c) += sum_{b <= a} C(a, b) (c' - c)^(a-b) M_b(c')      (child c')
 //   M2L  L_b(A) += sum_{|a|+|b| <= p} (-1)^|a| C(a+b, b) T_{a+b}(c_A - c_B) M_a(B)
 //   L2L  L_g(c') += sum_{b >= g} C(b, g) (c' - c)^(b-g) L_b(c)       (child c')
-//   L2P  phi_i += sum_b L_b (x_i - c)^b
+//   L2P  phi_i  = sum_b L_b (x_i - c)^b
 //   P2P  phi_i += sum_{j != i} q_j / |x_i - x_j|
 // with T_n = d^n(1/r)/n! from the recurrence in fmm_internal.h.  R is the
 // arithmetic type: double, or float for the mixed form, where the per-target
@@ -16,45 +16,14 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <type_traits>
 
+#include "fmm_arith.cuh"
 #include "fmm_internal.h"
 #include "scan.cuh"
 
 namespace gtap {
 namespace fmm {
 namespace {
-
-template <class R> struct Ops;
-template <> struct Ops<double> {
-    static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
-    static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-    static __device__ __forceinline__ double rsq(double a) { return rsqrt(a); }
-    static __device__ __forceinline__ double coef(const TermEntry& t) { return t.coef64; }
-};
-template <> struct Ops<float> {
-    static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
-    static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
-    static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ float rsq(float a) { return rsqrtf(a); }
-    static __device__ __forceinline__ float coef(const TermEntry& t) { return t.coef32; }
-};
-
-// Compensated accumulator (Kahan) for float; plain sum for double.
-template <class R> struct Acc {
-    R s = 0, c = 0;
-    __device__ __forceinline__ void add(R v) {
-        if constexpr (sizeof(R) == 4) {
-            const R y = Ops<R>::sub(v, c);
-            const R t = Ops<R>::add(s, y);
-            c = Ops<R>::sub(Ops<R>::sub(t, s), y);
-            s = t;
-        } else {
-            s += v;
-        }
-    }
-};
 
 // Index table (a, b, c) -> coefficient, (p+1)^3 shorts, in shared memory.
 __device__ __forceinline__ void load_index(const Tables& tb, short* idx) {
@@ -291,9 +260,6 @@ __global__ void k_m2l(EvalBufs e) {
 // 49 coefficients (plus 15 sums for z = 2) instead of 84.
 // The order P is a template parameter so that every index is a constant and
 // the compiler keeps Tt and Lt in registers.
-__host__ __device__ constexpr int cidx(int a, int b, int c) {
-    return (a + b + c) * (a + b + c + 1) * (a + b + c + 2) / 6 + (b + c) * (b + c + 1) / 2 + c;
-}
 // coefficients with z in {0, 1}: order k starts at k^2, its z = 0 entries by y, then z = 1 by y
 __host__ __device__ constexpr int n_harm(int p) { return (p + 1) * (p + 1); }
 __host__ __device__ constexpr int hidx(int a, int b, int c) {
@@ -551,237 +517,6 @@ __global__ void k_l2l(EvalBufs e, int lo, int hi) {
     }
 }
 
-// Packed FP32 pairs (two lanes of a 64-bit register) for the P2P inner loop:
-// one f32x2 instruction does the work of two FP32 ones.
-__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-    return (unsigned long long)__float_as_uint(lo) | ((unsigned long long)__float_as_uint(hi) << 32);
-}
-__device__ __forceinline__ float lo_f32(unsigned long long v) { return __uint_as_float((unsigned)v); }
-__device__ __forceinline__ float hi_f32(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
-__device__ __forceinline__ unsigned long long sub_f32x2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-// 1/sqrt(x), the hardware approximation (inputs here are normal: distinct points)
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// ---------------------------------------------------------------------------
-// Leaf kernel: one block per leaf.  Threads are (target slot, source part):
-// each thread sums over every parts-th source point of the near-field list,
-// source points staged in shared memory in batches of up to kSrcBatch from
-// consecutive source leaves; then the parts are combined and L2P added.
-constexpr int kLeafBlock = 128;
-constexpr int kSrcBatch = 1024;
-
-template <class R>
-__global__ void __launch_bounds__(kLeafBlock) k_leaf(EvalBufs e) {
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int p = e.p, nt = e.nt;
-    using R4 = typename std::conditional<sizeof(R) == 4, float4, Dbl4>::type;
-    R4* sp = reinterpret_cast<R4*>(sm_raw);             // [kSrcBatch] source x, y, z, q
-    int* sid = reinterpret_cast<int*>(sp + kSrcBatch);  // [kSrcBatch] sorted index
-    R* red = reinterpret_cast<R*>(sid + kSrcBatch);     // [kLeafBlock] (and a compensation array)
-    R* redc = red + kLeafBlock;
-    R* lsm = redc + kLeafBlock;                         // [nt]
-    int* bpre = reinterpret_cast<int*>(lsm + nt + (nt & 1));  // [33] prefix of the batch's source counts
-    int* bfirst = bpre + 34;                            // [32]
-    R* boff = reinterpret_cast<R*>(bfirst + 32);        // [32][3] source-centre offsets (mixed)
-    int* bnum = reinterpret_cast<int*>(boff + 96);      // [1]
-    short* idx = reinterpret_cast<short*>(bnum + 4);
-    load_index(e.tab, idx);
-    const int t = threadIdx.x, lane = t & 31;
-    for (int c = blockIdx.x; c < e.n_cells; c += gridDim.x) {
-        const int4 in = e.info[c];
-        if (in.z >= 0) continue;
-        const Dbl4 g = e.geom[c];
-        // one slot per target point, kLeafBlock / count source parts per slot
-        const int count = in.y;
-        const int tp = max(count, 1);
-        const int parts = kLeafBlock / tp;
-        const int part = t / tp, slot = t - part * tp;
-        const bool active = part < parts;
-        const int ki = in.x + (active ? slot : 0);
-        R xi, yi, zi;
-        if constexpr (sizeof(R) == 4) {
-            const float4 pl = e.ploc[ki];
-            xi = pl.x; yi = pl.y; zi = pl.z;
-        } else {
-            const Dbl4 pt = e.pts[ki];
-            xi = pt.x; yi = pt.y; zi = pt.z;
-        }
-        __syncthreads();
-        for (int i = t; i < nt; i += kLeafBlock) lsm[i] = (R)e.L[(size_t)c * nt + i];
-        Acc<R> acc;
-        if constexpr (sizeof(R) == 4) {
-            // the leaf's own points first: the target's own copy has exactly the same
-            // local coordinates (r^2 == 0) and is the only source that can, so only this
-            // pass tests for it; the batches below skip the leaf itself
-            __syncthreads();
-            for (int i = t; i < count; i += kLeafBlock) sp[i] = e.ploc[in.x + i];
-            __syncthreads();
-            if (active) {
-                float bsum = 0.f;
-                for (int j = part; j < count; j += parts) {
-                    const float4 sj = sp[j];
-                    const float dx = xi - sj.x, dy = yi - sj.y, dz = zi - sj.z;
-                    const float r2 = dx * dx + dy * dy + dz * dz;
-                    bsum += (r2 > 0.f) ? sj.w * rsqrtf(r2) : 0.f;
-                }
-                acc.add(bsum);
-            }
-        }
-        const int s0 = e.p2p_off[c], s1 = e.p2p_off[c + 1];
-        int cur = s0;
-        while (cur < s1) {
-            __syncthreads();
-            if (t < 32) {
-                const int j = cur + lane;
-                int cnt = 0, first = 0;
-                Dbl4 gs = make_dbl4(0, 0, 0, 0);
-                if (j < s1) {
-                    const int sc = e.p2p_src[j];
-                    const int4 si = e.info[sc];
-                    cnt = (sizeof(R) == 4 && sc == c) ? 0 : si.y;   // FP32: the own leaf had its pass
-                    first = si.x;
-                    gs = e.geom[sc];
-                }
-                int incl = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += y;
-                }
-                const unsigned fit = __ballot_sync(0xffffffffu, j < s1 && incl <= kSrcBatch);
-                const int nfit = max(1, __popc(fit));   // fit is a prefix of lanes; a leaf holds <= 64 points
-                if (lane < nfit) {
-                    bpre[lane + 1] = incl;
-                    bfirst[lane] = first;
-                    if constexpr (sizeof(R) == 4) {
-                        boff[lane * 3 + 0] = (R)__dsub_rn(gs.x, g.x);
-                        boff[lane * 3 + 1] = (R)__dsub_rn(gs.y, g.y);
-                        boff[lane * 3 + 2] = (R)__dsub_rn(gs.z, g.z);
-                    }
-                }
-                if (lane == 0) { bpre[0] = 0; bnum[0] = nfit; }
-            }
-            __syncthreads();
-            const int nfit = bnum[0];
-            const int total = bpre[nfit];
-            if constexpr (sizeof(R) == 4) {
-                // pair records {x0 x1 | y0 y1 | z0 z1 | q0 q1} of source points 2m, 2m+1
-                // (an odd tail is padded with a far, chargeless point)
-                float4* pr = reinterpret_cast<float4*>(sp);
-                for (int m = t; 2 * m < total; m += kLeafBlock) {
-                    const int i0 = 2 * m;
-                    int a = 0, b = nfit - 1;   // last source leaf with bpre[s] <= i0
-                    while (a < b) {
-                        const int mid = (a + b + 1) >> 1;
-                        if (bpre[mid] <= i0) a = mid; else b = mid - 1;
-                    }
-                    const float4 l0 = e.ploc[bfirst[a] + (i0 - bpre[a])];
-                    const float4 p0 = make_float4(l0.x + boff[a * 3], l0.y + boff[a * 3 + 1], l0.z + boff[a * 3 + 2], l0.w);
-                    float4 p1 = make_float4(1e18f, 1e18f, 1e18f, 0.f);
-                    if (i0 + 1 < total) {
-                        int a1 = a;   // skips empty entries (the target's own leaf counts 0 here)
-                        while (a1 + 1 < nfit && bpre[a1 + 1] <= i0 + 1) ++a1;
-                        const float4 l1 = e.ploc[bfirst[a1] + (i0 + 1 - bpre[a1])];
-                        p1 = make_float4(l1.x + boff[a1 * 3], l1.y + boff[a1 * 3 + 1], l1.z + boff[a1 * 3 + 2], l1.w);
-                    }
-                    pr[2 * m] = make_float4(p0.x, p1.x, p0.y, p1.y);
-                    pr[2 * m + 1] = make_float4(p0.z, p1.z, p0.w, p1.w);
-                }
-            } else {
-                for (int i = t; i < total; i += kLeafBlock) {
-                    int a = 0, b = nfit - 1;   // last source leaf with bpre[s] <= i
-                    while (a < b) {
-                        const int mid = (a + b + 1) >> 1;
-                        if (bpre[mid] <= i) a = mid; else b = mid - 1;
-                    }
-                    const int k = bfirst[a] + (i - bpre[a]);
-                    sid[i] = k;
-                    sp[i] = e.pts[k];
-                }
-            }
-            __syncthreads();
-            if (active) {
-                if constexpr (sizeof(R) == 4) {
-                    // other leaves only: no self term.  Two source points per step in
-                    // packed FP32 pairs; each batch is summed plainly and added to the
-                    // compensated total
-                    const unsigned long long X2 = pack_f32x2(xi, xi), Y2 = pack_f32x2(yi, yi), Z2 = pack_f32x2(zi, zi);
-                    const ulonglong2* pr = reinterpret_cast<const ulonglong2*>(sp);
-                    const int npairs = (total + 1) >> 1;
-                    unsigned long long acc2 = 0ull;
-#pragma unroll 2
-                    for (int m = part; m < npairs; m += parts) {
-                        const ulonglong2 xy = pr[2 * m], zq = pr[2 * m + 1];
-                        const unsigned long long dx = sub_f32x2(X2, xy.x), dy = sub_f32x2(Y2, xy.y), dz = sub_f32x2(Z2, zq.x);
-                        unsigned long long r2 = mul_f32x2(dx, dx);
-                        r2 = fma_f32x2(dy, dy, r2);
-                        r2 = fma_f32x2(dz, dz, r2);
-                        const unsigned long long ir = pack_f32x2(rsqrt_ftz(lo_f32(r2)), rsqrt_ftz(hi_f32(r2)));
-                        acc2 = fma_f32x2(zq.y, ir, acc2);
-                    }
-                    acc.add(lo_f32(acc2) + hi_f32(acc2));
-                } else {
-                    for (int j = part; j < total; j += parts) {
-                        if (sid[j] == ki) continue;
-                        const R4 s = sp[j];
-                        const R dx = xi - s.x, dy = yi - s.y, dz = zi - s.z;
-                        const R r2 = dx * dx + dy * dy + dz * dz;
-                        acc.add(s.w * Ops<R>::rsq(r2));
-                    }
-                }
-            }
-            cur += nfit;
-        }
-        red[t] = acc.s;
-        redc[t] = acc.c;
-        __syncthreads();
-        if (part == 0 && active) {
-            Acc<R> tot;
-            tot.s = red[t];
-            tot.c = redc[t];
-            for (int q = 1; q < parts; ++q) tot.add(Ops<R>::sub(red[q * tp + slot], redc[q * tp + slot]));
-            // L2P
-            R pl = 0;
-            const int p1 = p + 1;
-            R xa = 1;
-            const R dx = (sizeof(R) == 4) ? xi : (R)__dsub_rn((double)xi, g.x);
-            const R dy = (sizeof(R) == 4) ? yi : (R)__dsub_rn((double)yi, g.y);
-            const R dz = (sizeof(R) == 4) ? zi : (R)__dsub_rn((double)zi, g.z);
-            for (int a = 0; a <= p; ++a) {
-                R xab = xa;
-                for (int b = 0; a + b <= p; ++b) {
-                    R m = xab;
-                    for (int cc = 0; a + b + cc <= p; ++cc) {
-                        pl += lsm[idx[(a * p1 + b) * p1 + cc]] * m;
-                        m *= dz;
-                    }
-                    xab *= dy;
-                }
-                xa *= dx;
-            }
-            e.phi[e.order[ki]] = (double)tot.s - (double)tot.c + (double)pl;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Counting sort of a list by target.  The traversal appends the child pairs of
 // one split pair together, so a warp's 32 entries often share a target: the
@@ -831,13 +566,6 @@ template <class R>
 size_t m2l_smem(int p, int nt, int items) {
     return sizeof(R) * (2 * kSB * nt + 4 * kSB + items + 2 * (p + 1) + ((p + 1) & 1) + 2) + sizeof(DerivEntry) * nt + 16;
 }
-template <class R>
-size_t leaf_smem(int p, int nt) {
-    const size_t r4 = (sizeof(R) == 4) ? sizeof(float4) : sizeof(Dbl4);
-    return r4 * kSrcBatch + sizeof(int) * kSrcBatch + sizeof(R) * (2 * kLeafBlock + nt + (nt & 1)) + sizeof(int) * 66 +
-           sizeof(R) * 96 + sizeof(int) * 4 + sizeof(short) * (p + 1) * (p + 1) * (p + 1) + 16;
-}
-
 template <class K>
 cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -943,21 +671,6 @@ cudaError_t launch_downward(const EvalBufs& e, bool mixed, int fp64_levels, cuda
         if (err != cudaSuccess) return err;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_leaf_eval(const EvalBufs& e, bool mixed, cudaStream_t s) {
-    cudaError_t err;
-    const int grid = grid_for(e.n_cells, 1, 1 << 20);
-    if (mixed) {
-        const size_t sm = leaf_smem<float>(e.p, e.nt);
-        if ((err = set_smem(k_leaf<float>, sm)) != cudaSuccess) return err;
-        k_leaf<float><<<grid, kLeafBlock, sm, s>>>(e);
-    } else {
-        const size_t sm = leaf_smem<double>(e.p, e.nt);
-        if ((err = set_smem(k_leaf<double>, sm)) != cudaSuccess) return err;
-        k_leaf<double><<<grid, kLeafBlock, sm, s>>>(e);
-    }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_group(const unsigned long long* list, long long count, int n_cells, int* cnt, int* off, int* cursor,

@@ -186,7 +186,10 @@ size_t m2l_scratch_bytes(int p, int n_cells, bool mixed);
 cudaError_t launch_upward(const EvalBufs& e, bool mixed, int fp64_levels, cudaStream_t s);
 cudaError_t launch_m2l(const EvalBufs& e, bool mixed, cudaStream_t s);
 cudaError_t launch_downward(const EvalBufs& e, bool mixed, int fp64_levels, cudaStream_t s);
-cudaError_t launch_leaf_eval(const EvalBufs& e, bool mixed, cudaStream_t s);
+// P2P over the n_p2p entries of the grouped near lists, then L2P (fmm_leaf.cu).
+cudaError_t launch_leaf_eval(const EvalBufs& e, bool mixed, long long n_p2p, int n_leaves, int sms, void* scratch,
+                             cudaStream_t s);
+size_t p2p_scratch_bytes(bool mixed, long long n, long long n_p2p, int n_leaves, int sms);
 // Group list entries (target << 32 | source) by target: off[n_cells + 1], src[count].
 cudaError_t launch_group(const unsigned long long* list, long long count, int n_cells, int* cnt, int* off,
                          int* cursor, int* src, int* tile_sums, cudaStream_t s);
