@@ -478,6 +478,8 @@ def _fmm_levels_refined(n_levels: int) -> int:
 
 
 def _fmm_kernels_per_instance(n_levels: int, mixed: bool) -> int:
+    """Kernels of an instance with five launches per radix pass and per level; the count of the
+    present build is _fmm_launches_per_instance."""
     done = _fmm_levels_refined(n_levels)
     # bbox (2), codes, 8 radix passes (histogram, 3-kernel scan, scatter), 5 kernels per refined level,
     # level-start tail when stopped early, gather, record check, leaf-local coordinates (mixed)
@@ -485,6 +487,16 @@ def _fmm_kernels_per_instance(n_levels: int, mixed: bool) -> int:
     upward = 1 + max(n_levels - 1, 0)
     traverse = 2
     evaluate = 2 * 5 + 2 + max(n_levels - 1, 0) + 1
+    return tree + upward + traverse + evaluate
+
+
+def _fmm_launches_per_instance(n_levels: int, mixed: bool) -> int:
+    # bounding box, codes, 8 radix passes, refinement, gather, record check, leaf-local coordinates (mixed)
+    tree = 2 + 8 + 1 + 1 + 1 + (1 if mixed else 0)
+    upward = 1 + max(n_levels - 1, 0)
+    traverse = 2
+    # two list groupings, multipole folding and M2L, L2L levels, near-field runs, P2P and L2P
+    evaluate = 2 * 5 + 2 + max(n_levels - 1, 0) + 3
     return tree + upward + traverse + evaluate
 
 
@@ -587,7 +599,7 @@ def run_fmm(args):
     else:
         peak = FP64_NOMINAL_TFLOPS
         peak_kind = "nominal GB300 FP64"
-    launches = sum(_fmm_kernels_per_instance(info[dd]["n_levels"], mixed) for dd in sets) * args.steps
+    launches = sum(_fmm_launches_per_instance(info[dd]["n_levels"], mixed) for dd in sets) * args.steps
     m2l_traffic = None
     if mixed:
         try:

@@ -155,8 +155,8 @@ struct gtap_fmm {
     DBuf tab_dev;
 
     // tree
-    DBuf keys0, keys1, vals0, vals1, pts, ploc, hist, hist_scan, tile_sums, box, bbox_part, geom, info, lat, lstart,
-        lvl_n, lvl_total, cnt, off, bounds, flags;
+    DBuf keys0, keys1, vals0, vals1, pts, ploc, work, tile_sums, block_sums, box, bbox_part, geom, info, lat, lstart,
+        bounds, flags;
     double box_h[8] = {};
     int cell_cap = 0;
     const uint32_t* order = nullptr;
@@ -173,8 +173,8 @@ struct gtap_fmm {
     cudaEvent_t ev[8] = {};
 
     ~gtap_fmm() {
-        DBuf* all[] = {&tab_dev, &keys0, &keys1, &vals0, &vals1, &pts, &ploc, &hist, &hist_scan, &tile_sums, &box,
-                       &bbox_part, &geom, &info, &lat, &lstart, &lvl_n, &lvl_total, &cnt, &off, &bounds, &flags, &M, &L,
+        DBuf* all[] = {&tab_dev, &keys0, &keys1, &vals0, &vals1, &pts, &ploc, &work, &tile_sums, &block_sums, &box,
+                       &bbox_part, &geom, &info, &lat, &lstart, &bounds, &flags, &M, &L,
                        &m2l, &p2p, &counters, &gcnt, &gcur, &m2l_off, &m2l_src, &p2p_off, &p2p_src, &p2p_runs, &ms, &aux};
         for (DBuf* b : all) b->release();
         for (cudaEvent_t& e : ev)
@@ -321,7 +321,7 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
     if (!f->counters.ensure(4 * sizeof(unsigned long long)) || !f->aux.ensure(sizeof(DttAux)) ||
         !f->box.ensure(8 * sizeof(double)) ||
         !f->bbox_part.ensure(6 * kBoxParts * sizeof(double)) || !f->lstart.ensure((kMaxLevel + 3) * sizeof(int)) ||
-        !f->lvl_n.ensure((kMaxLevel + 1) * sizeof(int)) || !f->lvl_total.ensure((kMaxLevel + 1) * sizeof(int)) ||
+        !f->block_sums.ensure(sizeof(int) * (size_t)f->sms) ||
         !f->flags.ensure(4 * sizeof(int))) {
         delete f;
         return GTAP_ERR_NO_MEMORY;
@@ -334,10 +334,8 @@ gtap_status gtap_fmm_build(gtap_fmm* f, const double* pos, const double* q, int6
     if (!f || !pos || !q || n < 1 || n >= (1ll << 31) - 1) return GTAP_ERR_INVALID_ARG;
     f->built = f->traversed = false;
     const size_t N = (size_t)n;
-    const int ntiles = radix_tiles(n);
     if (!f->keys0.ensure(8 * N) || !f->keys1.ensure(8 * N) || !f->vals0.ensure(4 * N) || !f->vals1.ensure(4 * N) ||
-        !f->pts.ensure(sizeof(Dbl4) * N) || !f->hist.ensure(sizeof(int) * 256 * (size_t)ntiles) ||
-        !f->hist_scan.ensure(sizeof(int) * 256 * (size_t)ntiles) || (f->mixed && !f->ploc.ensure(sizeof(float4) * N)))
+        !f->pts.ensure(sizeof(Dbl4) * N) || !f->work.ensure(tree_work_bytes(n)) || (f->mixed && !f->ploc.ensure(sizeof(float4) * N)))
         return GTAP_ERR_NO_MEMORY;
     // cell capacity: a first guess, doubled while a level does not fit
     long long cap = std::max<long long>(1024, 2 * (8 * n / (f->cfg.leaf_size + 1)) + 64);
@@ -347,9 +345,7 @@ gtap_status gtap_fmm_build(gtap_fmm* f, const double* pos, const double* q, int6
         if (cap >= (1ll << 31) / 9) return GTAP_ERR_NO_MEMORY;
         const size_t C = (size_t)cap;
         if (!f->geom.ensure(sizeof(Dbl4) * C) || !f->info.ensure(sizeof(int4) * C) || !f->lat.ensure(sizeof(int4) * C) ||
-            !f->cnt.ensure(sizeof(int) * C) ||
-            !f->off.ensure(sizeof(int) * C) || !f->bounds.ensure(sizeof(int) * 9 * C) ||
-            !f->tile_sums.ensure(sizeof(int) * (size_t)scan::tiles_for(std::max<long long>(cap, 256ll * ntiles))))
+            !f->bounds.ensure(sizeof(int) * 9 * C))
             return GTAP_ERR_NO_MEMORY;
         f->cell_cap = (int)cap;
         TreeBufs b{};
@@ -363,40 +359,18 @@ gtap_status gtap_fmm_build(gtap_fmm* f, const double* pos, const double* q, int6
         b.keys[1] = f->keys1.as<unsigned long long>();
         b.vals[0] = f->vals0.as<uint32_t>();
         b.vals[1] = f->vals1.as<uint32_t>();
-        b.hist = f->hist.as<int>();
-        b.hist_scan = f->hist_scan.as<int>();
-        b.tile_sums = f->tile_sums.as<int>();
+        b.work = f->work.p;
+        b.block_sums = f->block_sums.as<int>();
         b.geom = f->geom.as<Dbl4>();
         b.info = f->info.as<int4>();
         b.lat = f->lat.as<int4>();
         b.cap_cells = (int)cap;
         b.lstart = f->lstart.as<int>();
-        b.lvl_n = f->lvl_n.as<int>();
-        b.lvl_total = f->lvl_total.as<int>();
-        b.cnt = f->cnt.as<int>();
-        b.off = f->off.as<int>();
         b.bounds = f->bounds.as<int>();
         b.flags = f->flags.as<int>();
         b.pts = f->pts.as<Dbl4>();
         b.ploc = f->ploc.as<float4>();
-        if (launch_tree_sort(b, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
-        // Refine level by level.  A level without cells ends the tree, so between
-        // chunks of levels the host looks at the next level's size and stops at the
-        // first empty one (a uniform 2^20 set has 6 levels, a Plummer set 10, of 21).
-        int done = 0;
-        for (int chunk : {8, 4, 4, 5}) {
-            const int l1 = std::min(done + chunk, kMaxLevel);
-            if (launch_tree_levels(b, done, l1, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
-            done = l1;
-            if (done >= kMaxLevel) break;
-            int ls[2] = {0, 0};   // the cells of level `done`: [ls[0], ls[1])
-            if (cudaMemcpyAsync(ls, f->lstart.as<int>() + done, sizeof(ls), cudaMemcpyDeviceToHost, f->s) !=
-                    cudaSuccess ||
-                cudaStreamSynchronize(f->s) != cudaSuccess)
-                return GTAP_ERR_CUDA;
-            if (ls[1] == ls[0]) break;
-        }
-        if (launch_tree_finish(b, done, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
+        if (launch_tree(b, f->sms, f->s) != cudaSuccess) return GTAP_ERR_CUDA;
         int flags[4] = {0, 0, 0, 0};
         if (cudaMemcpyAsync(flags, f->flags.p, sizeof(flags), cudaMemcpyDeviceToHost, f->s) != cudaSuccess ||
             cudaMemcpyAsync(f->lstart_h, f->lstart.p, sizeof(f->lstart_h), cudaMemcpyDeviceToHost, f->s) != cudaSuccess ||

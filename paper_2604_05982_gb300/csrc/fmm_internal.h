@@ -127,18 +127,13 @@ struct TreeBufs {
     double* bbox_part;            // [6 * kBoxParts]
     unsigned long long* keys[2];  // radix-sort ping-pong
     uint32_t* vals[2];
-    int* hist;                    // [256 * ntiles]
-    int* hist_scan;
-    int* tile_sums;               // scan scratch
+    void* work;                   // tree_work_bytes(n): counters, digit counts, look-back words
+    int* block_sums;              // [SM count]: children per block of the refinement
     Dbl4* geom;
     int4* info;
     int4* lat;                    // cell centre on the level-21 lattice: (2i+1) << (21 - level) per axis, level
     int cap_cells;
     int* lstart;                  // [kMaxLevel + 3]: first cell of each level
-    int* lvl_n;                   // [kMaxLevel + 1]: cells per level
-    int* lvl_total;               // [kMaxLevel + 1]: children created per level
-    int* cnt;                     // [cap_cells] per-level child counts
-    int* off;                     // [cap_cells] their exclusive scan
     int* bounds;                  // [9 * cap_cells] octant boundaries
     int* flags;                   // [4]: [0] cell capacity exceeded, [1] malformed record, [2] leaves, [3] largest leaf
     Dbl4* pts;                 // sorted points {x, y, z, q}
@@ -148,14 +143,11 @@ struct TreeBufs {
 };
 constexpr int kBoxParts = 304;
 
-int radix_tiles(long long n);
-// Tree build in three stream-ordered parts: bounding box, Morton codes and
-// radix sort; refinement of levels [l0, l1); then the start entries of levels
-// left unrefined (all empty), the gather of points into tree order, and the
+size_t tree_work_bytes(long long n);
+// Tree build, stream-ordered: bounding box, Morton codes and radix sort;
+// refinement of all levels; the gather of points into tree order, and the
 // structural check of the cell records (flags[1..3]).
-cudaError_t launch_tree_sort(TreeBufs& b, cudaStream_t s);
-cudaError_t launch_tree_levels(const TreeBufs& b, int l0, int l1, cudaStream_t s);
-cudaError_t launch_tree_finish(const TreeBufs& b, int levels_done, cudaStream_t s);
+cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s);
 // Leaf-local FP32 coordinates (needs the cell count, known after the build).
 cudaError_t launch_leaf_local(const TreeBufs& b, int n_cells, cudaStream_t s);
 
