@@ -51,9 +51,10 @@ struct HostTables {
     std::vector<DerivEntry> deriv;
     std::vector<ItemEntry> items;
     std::vector<int> item_off;
-    std::vector<TermEntry> m2l, m2m, l2l;
+    std::vector<TermEntry> m2l;
+    std::vector<uint32_t> m2m, l2l;
     std::vector<int> m2m_off, l2l_off;
-    std::vector<double> mscale, lscale;   // (-1)^|a| / a!  and  1 / b!  per coefficient
+    std::vector<double> mscale, lscale, fact;   // (-1)^|a| / a!,  1 / b!  and  b!  per coefficient
 
     int at(int a, int b, int c) const {
         if (a < 0 || b < 0 || c < 0 || a + b + c > p) return -1;
@@ -88,6 +89,7 @@ struct HostTables {
             for (int t = 2; t <= a; ++t) fa *= t;
             for (int t = 2; t <= b; ++t) fa *= t;
             for (int t = 2; t <= c; ++t) fa *= t;
+            fact.push_back(fa);
             lscale.push_back(1.0 / fa);
             mscale.push_back(((a + b + c) & 1) ? -1.0 / fa : 1.0 / fa);
         }
@@ -122,11 +124,9 @@ struct HostTables {
             for (int bi = 0; bi < nt; ++bi) {
                 const short3 be = mi[bi];
                 if (be.x <= al.x && be.y <= al.y && be.z <= al.z)
-                    m2m.push_back(term(bi, at(al.x - be.x, al.y - be.y, al.z - be.z),
-                                       binom(al.x, be.x) * binom(al.y, be.y) * binom(al.z, be.z)));
+                    m2m.push_back((uint32_t)bi | (uint32_t)at(al.x - be.x, al.y - be.y, al.z - be.z) << 16);
                 if (be.x >= al.x && be.y >= al.y && be.z >= al.z)
-                    l2l.push_back(term(bi, at(be.x - al.x, be.y - al.y, be.z - al.z),
-                                       binom(be.x, al.x) * binom(be.y, al.y) * binom(be.z, al.z)));
+                    l2l.push_back((uint32_t)bi | (uint32_t)at(be.x - al.x, be.y - al.y, be.z - al.z) << 16);
             }
         }
         m2m_off.push_back((int)m2m.size());
@@ -289,7 +289,7 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
     const size_t o_mi = put(blob, h.mi), o_der = put(blob, h.deriv), o_items = put(blob, h.items),
                  o_ioff = put(blob, h.item_off), o_m2l = put(blob, h.m2l), o_m2mo = put(blob, h.m2m_off),
                  o_m2m = put(blob, h.m2m), o_l2lo = put(blob, h.l2l_off), o_l2l = put(blob, h.l2l),
-                 o_ms = put(blob, h.mscale), o_ls = put(blob, h.lscale);
+                 o_ms = put(blob, h.mscale), o_ls = put(blob, h.lscale), o_fa = put(blob, h.fact);
     if (!f->tab_dev.ensure(blob.size()) ||
         cudaMemcpy(f->tab_dev.p, blob.data(), blob.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         delete f;
@@ -301,18 +301,18 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
     t.nt = f->nt;
     t.n_m2l_items = (int)h.items.size();
     t.n_m2l_terms = (int)h.m2l.size();
-    t.n_shift_terms = (int)h.m2m.size();
     t.mi = reinterpret_cast<short3*>(base + o_mi);
     t.deriv = reinterpret_cast<DerivEntry*>(base + o_der);
     t.m2l_items = reinterpret_cast<ItemEntry*>(base + o_items);
     t.m2l_item_off = reinterpret_cast<int*>(base + o_ioff);
     t.m2l_terms = reinterpret_cast<TermEntry*>(base + o_m2l);
     t.m2m_off = reinterpret_cast<int*>(base + o_m2mo);
-    t.m2m_terms = reinterpret_cast<TermEntry*>(base + o_m2m);
+    t.m2m_terms = reinterpret_cast<uint32_t*>(base + o_m2m);
     t.l2l_off = reinterpret_cast<int*>(base + o_l2lo);
-    t.l2l_terms = reinterpret_cast<TermEntry*>(base + o_l2l);
+    t.l2l_terms = reinterpret_cast<uint32_t*>(base + o_l2l);
     t.mscale = reinterpret_cast<double*>(base + o_ms);
     t.lscale = reinterpret_cast<double*>(base + o_ls);
+    t.fact = reinterpret_cast<double*>(base + o_fa);
     for (cudaEvent_t& e : f->ev)
         if (cudaEventCreate(&e) != cudaSuccess) {
             delete f;

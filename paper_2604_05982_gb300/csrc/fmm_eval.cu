@@ -25,36 +25,41 @@ namespace gtap {
 namespace fmm {
 namespace {
 
-// Index table (a, b, c) -> coefficient, (p+1)^3 shorts, in shared memory.
-__device__ __forceinline__ void load_index(const Tables& tb, short* idx) {
-    const int p1 = tb.p + 1;
-    for (int i = threadIdx.x; i < p1 * p1 * p1; i += blockDim.x) idx[i] = -1;
-    __syncthreads();
-    for (int i = threadIdx.x; i < tb.nt; i += blockDim.x) {
-        const short3 m = tb.mi[i];
-        idx[(m.x * p1 + m.y) * p1 + m.z] = (short)i;
+// M2M and L2L between a cell and its children work in the scaled variables
+// M_a / a!, b! L_b and d^n / n!, where a shift is a plain correlation: one
+// multiply-add per term, no binomials.  One warp per child, a lane per output
+// coefficient; the displacement's scaled monomials come from three short power
+// tables.  One thread per coefficient for all eight children, binomials read
+// with every term and the monomials built by one thread per child took 25 us a
+// level, whatever its size; a small set's passes are bound by that chain.
+constexpr int kShiftBlock = 256;   // 8 warps
+
+// Scaled powers d_x^k / k! of every child's displacement: pw[child][axis][k].
+template <class R>
+__device__ __forceinline__ void shift_powers(const EvalBufs& e, const Dbl4& g, int cf, int nch, R* pw) {
+    const int t = threadIdx.x, j = t / 3, axis = t % 3, p1 = kMaxOrder + 1;
+    if (j < nch) {
+        const Dbl4 gc = e.geom[cf + j];
+        const R d = (R)(axis == 0 ? __dsub_rn(gc.x, g.x) : axis == 1 ? __dsub_rn(gc.y, g.y) : __dsub_rn(gc.z, g.z));
+        R v = 1;
+        pw[t * p1] = v;
+        for (int k = 1; k <= e.p; ++k) {
+            v = v * d / (R)k;
+            pw[t * p1 + k] = v;
+        }
     }
-    __syncthreads();
 }
 
-// Monomials x^a y^b z^c of one displacement for every coefficient, by the
-// nested powers (no table of powers needed).
+// Warp j fills mono[i] = d^n / n! of child j for every coefficient.
 template <class R>
-__device__ __forceinline__ void monomials(int p, const short* idx, R x, R y, R z, R* out) {
-    const int p1 = p + 1;
-    R xa = 1;
-    for (int a = 0; a <= p; ++a) {
-        R xab = xa;
-        for (int b = 0; a + b <= p; ++b) {
-            R t = xab;
-            for (int c = 0; a + b + c <= p; ++c) {
-                out[idx[(a * p1 + b) * p1 + c]] = t;
-                t = Ops<R>::mul(t, z);
-            }
-            xab = Ops<R>::mul(xab, y);
-        }
-        xa = Ops<R>::mul(xa, x);
+__device__ __forceinline__ void shift_monomials(const EvalBufs& e, const R* pw, R* mono) {
+    const int lane = threadIdx.x & 31, p1 = kMaxOrder + 1;
+    const R* w = pw + 3 * p1 * (threadIdx.x >> 5);
+    for (int i = lane; i < e.nt; i += 32) {
+        const short3 n = e.tab.mi[i];
+        mono[i] = w[n.x] * w[p1 + n.y] * w[2 * p1 + n.z];
     }
+    __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
@@ -104,43 +109,41 @@ __global__ void k_p2m(EvalBufs e) {
     }
 }
 
-// M2M for the parents of one level: one block per parent.
+// M2M for the parents of one level: one block per cell, leaves leave at once.
 template <class R>
-__global__ void k_m2m(EvalBufs e, int lo, int hi) {
+__global__ void __launch_bounds__(kShiftBlock) k_m2m(EvalBufs e, int lo) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int p = e.p, nt = e.nt, p1 = p + 1;
-    R* mono = reinterpret_cast<R*>(sm_raw);            // [8][nt]
-    R* mc = mono + 8 * nt;                             // [8][nt]
-    short* idx = reinterpret_cast<short*>(mc + 8 * nt);
-    load_index(e.tab, idx);
-    for (int c = lo + blockIdx.x; c < hi; c += gridDim.x) {
-        const int4 in = e.info[c];
-        if (in.z < 0) continue;
-        const int nch = in.w & 0xFF, cf = in.z;
-        const Dbl4 g = e.geom[c];
-        __syncthreads();
-        if ((int)threadIdx.x < nch) {
-            const Dbl4 gc = e.geom[cf + threadIdx.x];
-            monomials<R>(p, idx, (R)__dsub_rn(gc.x, g.x), (R)__dsub_rn(gc.y, g.y), (R)__dsub_rn(gc.z, g.z),
-                         mono + threadIdx.x * nt);
-        }
-        for (int i = threadIdx.x; i < nch * nt; i += blockDim.x) mc[i] = (R)e.M[(size_t)cf * nt + i];
-        __syncthreads();
-        for (int a = threadIdx.x; a < nt; a += blockDim.x) {
-            const int t0 = e.tab.m2m_off[a], t1 = e.tab.m2m_off[a + 1];
-            Acc<R> acc;
-            for (int j = 0; j < nch; ++j) {
-                R s = 0;
-                for (int t = t0; t < t1; ++t) {
-                    const TermEntry te = e.tab.m2m_terms[t];
-                    s += Ops<R>::coef(te) * mono[j * nt + te.b] * mc[j * nt + te.a];
-                }
-                acc.add(s);
+    const int nt = e.nt, c = lo + (int)blockIdx.x, t = threadIdx.x, lane = t & 31, j = t >> 5;
+    const int4 in = e.info[c];
+    if (in.z < 0) return;
+    const int nch = in.w & 0xFF, cf = in.z;
+    R* pw = reinterpret_cast<R*>(sm_raw);              // [8][3][kMaxOrder + 1]
+    R* mono = pw + 24 * (kMaxOrder + 1) + j * nt;      // [8][nt], this warp's row
+    R* mc = pw + 24 * (kMaxOrder + 1) + (8 + j) * nt;  // [8][nt]
+    R* part = pw + 24 * (kMaxOrder + 1) + 16 * nt;     // [8][nt]
+    shift_powers(e, e.geom[c], cf, nch, pw);
+    if (j < nch)
+        for (int i = lane; i < nt; i += 32) mc[i] = (R)(e.M[(size_t)(cf + j) * nt + i] * __ldg(e.tab.lscale + i));
+    __syncthreads();
+    if (j < nch) {
+        shift_monomials(e, pw, mono);
+        for (int a = lane; a < nt; a += 32) {
+            const int t1 = __ldg(e.tab.m2m_off + a + 1);
+            R s = 0;
+#pragma unroll 4
+            for (int i = __ldg(e.tab.m2m_off + a); i < t1; ++i) {
+                const unsigned u = __ldg(e.tab.m2m_terms + i);
+                s += mono[u >> 16] * mc[u & 0xFFFFu];
             }
-            e.M[(size_t)c * nt + a] = (double)acc.s - (double)acc.c;
+            part[j * nt + a] = s;
         }
     }
-    (void)p1;
+    __syncthreads();
+    for (int a = t; a < nt; a += kShiftBlock) {
+        Acc<R> acc;
+        for (int k = 0; k < nch; ++k) acc.add(part[k * nt + a]);
+        e.M[(size_t)c * nt + a] = ((double)acc.s - (double)acc.c) * __ldg(e.tab.fact + a);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -482,38 +485,31 @@ __global__ void __launch_bounds__(32 * kM2lWarps) k_m2l_reg64(EvalBufs e, const 
     m2l_finish<P>(L, T - lane, e, tgt);
 }
 
-// L2L from the parents of one level into their children: one block per parent.
+// L2L from the cells of one level into their children: one block per cell.
 template <class R>
-__global__ void k_l2l(EvalBufs e, int lo, int hi) {
+__global__ void __launch_bounds__(kShiftBlock) k_l2l(EvalBufs e, int lo) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int p = e.p, nt = e.nt;
-    R* mono = reinterpret_cast<R*>(sm_raw);            // [8][nt]
-    R* lp = mono + 8 * nt;                             // [nt]
-    short* idx = reinterpret_cast<short*>(lp + nt);
-    load_index(e.tab, idx);
-    for (int c = lo + blockIdx.x; c < hi; c += gridDim.x) {
-        const int4 in = e.info[c];
-        if (in.z < 0) continue;
-        const int nch = in.w & 0xFF, cf = in.z;
-        const Dbl4 g = e.geom[c];
-        __syncthreads();
-        if ((int)threadIdx.x < nch) {
-            const Dbl4 gc = e.geom[cf + threadIdx.x];
-            monomials<R>(p, idx, (R)__dsub_rn(gc.x, g.x), (R)__dsub_rn(gc.y, g.y), (R)__dsub_rn(gc.z, g.z),
-                         mono + threadIdx.x * nt);
+    const int nt = e.nt, c = lo + (int)blockIdx.x, t = threadIdx.x, lane = t & 31, j = t >> 5;
+    const int4 in = e.info[c];
+    if (in.z < 0) return;
+    const int nch = in.w & 0xFF, cf = in.z;
+    R* pw = reinterpret_cast<R*>(sm_raw);              // [8][3][kMaxOrder + 1]
+    R* lp = pw + 24 * (kMaxOrder + 1);                 // [nt]
+    R* mono = lp + nt + j * nt;                        // [8][nt], this warp's row
+    shift_powers(e, e.geom[c], cf, nch, pw);
+    for (int i = t; i < nt; i += kShiftBlock) lp[i] = (R)(e.L[(size_t)c * nt + i] * __ldg(e.tab.fact + i));
+    __syncthreads();
+    if (j >= nch) return;
+    shift_monomials(e, pw, mono);
+    for (int g = lane; g < nt; g += 32) {
+        const int t1 = __ldg(e.tab.l2l_off + g + 1);
+        R s = 0;
+#pragma unroll 4
+        for (int i = __ldg(e.tab.l2l_off + g); i < t1; ++i) {
+            const unsigned u = __ldg(e.tab.l2l_terms + i);
+            s += mono[u >> 16] * lp[u & 0xFFFFu];
         }
-        for (int i = threadIdx.x; i < nt; i += blockDim.x) lp[i] = (R)e.L[(size_t)c * nt + i];
-        __syncthreads();
-        for (int w = threadIdx.x; w < nch * nt; w += blockDim.x) {
-            const int j = w / nt, gi = w - j * nt;
-            const int t0 = e.tab.l2l_off[gi], t1 = e.tab.l2l_off[gi + 1];
-            R s = 0;
-            for (int t = t0; t < t1; ++t) {
-                const TermEntry te = e.tab.l2l_terms[t];
-                s += Ops<R>::coef(te) * mono[j * nt + te.b] * lp[te.a];
-            }
-            e.L[(size_t)(cf + j) * nt + gi] += (double)s;
-        }
+        e.L[(size_t)(cf + j) * nt + g] += (double)s * __ldg(e.tab.lscale + g);
     }
 }
 
@@ -559,9 +555,9 @@ int grid_for(long long n, int block, int cap) {
 template <class R>
 size_t p2m_smem(int p, int nt) { return sizeof(R) * (kMaxLeaf * 3 * (p + 1) + kMaxLeaf) + sizeof(short3) * nt + 16; }
 template <class R>
-size_t m2m_smem(int p, int nt) { return sizeof(R) * 16 * nt + sizeof(short) * (p + 1) * (p + 1) * (p + 1) + 16; }
+size_t m2m_smem(int nt) { return sizeof(R) * (24 * (kMaxOrder + 1) + 24 * nt); }
 template <class R>
-size_t l2l_smem(int p, int nt) { return sizeof(R) * 9 * nt + sizeof(short) * (p + 1) * (p + 1) * (p + 1) + 16; }
+size_t l2l_smem(int nt) { return sizeof(R) * (24 * (kMaxOrder + 1) + 9 * nt); }
 template <class R>
 size_t m2l_smem(int p, int nt, int items) {
     return sizeof(R) * (2 * kSB * nt + 4 * kSB + items + 2 * (p + 1) + ((p + 1) & 1) + 2) + sizeof(DerivEntry) * nt + 16;
@@ -574,22 +570,14 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 template <class R>
 cudaError_t upward_level(const EvalBufs& e, int l, cudaStream_t s) {
     const int lo = e.lstart[l], hi = e.lstart[l + 1];
-    if (hi <= lo) return cudaSuccess;
-    const size_t sm = m2m_smem<R>(e.p, e.nt);
-    cudaError_t err = set_smem(k_m2m<R>, sm);
-    if (err != cudaSuccess) return err;
-    k_m2m<R><<<grid_for(hi - lo, 1, 1 << 20), 128, sm, s>>>(e, lo, hi);
+    if (hi > lo) k_m2m<R><<<hi - lo, kShiftBlock, m2m_smem<R>(e.nt), s>>>(e, lo);   // at most 33 KB: no opt-in
     return cudaGetLastError();
 }
 
 template <class R>
 cudaError_t downward_level(const EvalBufs& e, int l, cudaStream_t s) {
     const int lo = e.lstart[l], hi = e.lstart[l + 1];
-    if (hi <= lo) return cudaSuccess;
-    const size_t sm = l2l_smem<R>(e.p, e.nt);
-    cudaError_t err = set_smem(k_l2l<R>, sm);
-    if (err != cudaSuccess) return err;
-    k_l2l<R><<<grid_for(hi - lo, 1, 1 << 20), 128, sm, s>>>(e, lo, hi);
+    if (hi > lo) k_l2l<R><<<hi - lo, kShiftBlock, l2l_smem<R>(e.nt), s>>>(e, lo);
     return cudaGetLastError();
 }
 

@@ -97,18 +97,19 @@ struct ItemEntry {        // a run of terms with one output coefficient
 
 struct Tables {
     int p, nt;
-    int n_m2l_items, n_m2l_terms, n_shift_terms;
+    int n_m2l_items, n_m2l_terms;
     short3* mi;                 // (a, b, c) per coefficient
     DerivEntry* deriv;
     ItemEntry* m2l_items;
     int* m2l_item_off;          // [nt + 1]: items of output coefficient beta (items are sorted by beta)
     TermEntry* m2l_terms;       // a = alpha (index into M), b = alpha + beta (index into T)
     int* m2m_off;               // [nt + 1] offsets into m2m_terms, by alpha
-    TermEntry* m2m_terms;       // a = beta (index into child M), b = alpha - beta (monomial index)
+    uint32_t* m2m_terms;        // beta (index into child M) | (alpha - beta: monomial index) << 16
     int* l2l_off;               // [nt + 1] by gamma
-    TermEntry* l2l_terms;       // a = beta (index into parent L), b = beta - gamma (monomial index)
+    uint32_t* l2l_terms;        // beta (index into parent L) | (beta - gamma: monomial index) << 16
     double* mscale;             // [nt] (-1)^|alpha| / alpha!  (scaled multipoles of the M2L)
-    double* lscale;             // [nt] 1 / beta!  (local coefficients from the scaled M2L sums)
+    double* lscale;             // [nt] 1 / beta!  (local coefficients from the scaled sums)
+    double* fact;               // [nt] beta!
 };
 
 }  // namespace fmm
