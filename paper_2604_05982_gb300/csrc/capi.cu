@@ -91,9 +91,14 @@ struct gtap_ctx {
     RootDesc* root_desc_pinned = nullptr;
     int* host_abort = nullptr;       // pinned, mapped
     int* host_abort_dev = nullptr;
-    DevControl* ctl_pinned = nullptr;
-    RootEntry* roots_pinned = nullptr;
-    WorkerStats* stats_pinned = nullptr;
+    RunReport* report = nullptr;     // pinned, mapped: written by the report kernel
+    RunReport* report_dev = nullptr;
+    RootEntry* roots_pinned = nullptr;   // pinned, mapped
+    RootEntry* roots_pinned_dev = nullptr;
+    // the occupancy of the kernel last launched (asking the runtime costs microseconds a run)
+    unsigned occ_pset = 0;
+    size_t occ_smem = 0;
+    int occ_blocks = 0;
 
     std::vector<RootDesc> pending_roots;
     unsigned registered = 0;
@@ -110,7 +115,6 @@ struct gtap_ctx {
     cudaEvent_t ev_k0 = nullptr, ev_k1 = nullptr;         // the persistent kernel alone
     gtap_stats last_stats{};
     gtap_error_info last_err{};
-    bool cq_initialised = false;
     // CUDA-graph replay of a captured run
     cudaStream_t own_stream = nullptr;
     cudaGraph_t graph = nullptr;
@@ -130,6 +134,10 @@ struct gtap_ctx {
     HostFlags* hflags_dev = nullptr;
     uint64_t submitted = 0;
 };
+
+namespace gtap {
+cudaStream_t ctx_stream(const gtap_ctx* c) { return c->stream; }
+}  // namespace gtap
 
 extern "C" {
 
@@ -168,9 +176,8 @@ static gtap_status free_all(gtap_ctx* c) {
     if (c->own_arena && c->arena) cudaFree(c->arena);
     if (c->root_desc_pinned) cudaFreeHost(c->root_desc_pinned);
     if (c->host_abort) cudaFreeHost(c->host_abort);
-    if (c->ctl_pinned) cudaFreeHost(c->ctl_pinned);
+    if (c->report) cudaFreeHost(c->report);
     if (c->roots_pinned) cudaFreeHost(c->roots_pinned);
-    if (c->stats_pinned) cudaFreeHost(c->stats_pinned);
     if (c->ev_start) cudaEventDestroy(c->ev_start);
     if (c->ev_stop) cudaEventDestroy(c->ev_stop);
     if (c->ev_k0) cudaEventDestroy(c->ev_k0);
@@ -352,9 +359,10 @@ gtap_status gtap_init(gtap_mode mode, int n_queues, size_t frame_pool_bytes, con
     bool ok = cudaHostAlloc(reinterpret_cast<void**>(&c->root_desc_pinned), (size_t)cfg.max_roots * sizeof(RootDesc), cudaHostAllocDefault) == cudaSuccess &&
               cudaHostAlloc(reinterpret_cast<void**>(&c->host_abort), 128, cudaHostAllocMapped) == cudaSuccess &&
               cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->host_abort_dev), c->host_abort, 0) == cudaSuccess &&
-              cudaHostAlloc(reinterpret_cast<void**>(&c->ctl_pinned), sizeof(DevControl), cudaHostAllocDefault) == cudaSuccess &&
-              cudaHostAlloc(reinterpret_cast<void**>(&c->roots_pinned), (size_t)cfg.max_roots * sizeof(RootEntry), cudaHostAllocDefault) == cudaSuccess &&
-              cudaHostAlloc(reinterpret_cast<void**>(&c->stats_pinned), (size_t)c->n_workers_max * sizeof(WorkerStats), cudaHostAllocDefault) == cudaSuccess &&
+              cudaHostAlloc(reinterpret_cast<void**>(&c->report), sizeof(RunReport), cudaHostAllocMapped) == cudaSuccess &&
+              cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->report_dev), c->report, 0) == cudaSuccess &&
+              cudaHostAlloc(reinterpret_cast<void**>(&c->roots_pinned), (size_t)cfg.max_roots * sizeof(RootEntry), cudaHostAllocMapped) == cudaSuccess &&
+              cudaHostGetDevicePointer(reinterpret_cast<void**>(&c->roots_pinned_dev), c->roots_pinned, 0) == cudaSuccess &&
               cudaEventCreate(&c->ev_start) == cudaSuccess && cudaEventCreate(&c->ev_stop) == cudaSuccess &&
               cudaEventCreate(&c->ev_k0) == cudaSuccess && cudaEventCreate(&c->ev_k1) == cudaSuccess;
     if (!ok) {
@@ -623,6 +631,23 @@ gtap_status gtap_capture_graph(gtap_ctx* c) {
     return GTAP_OK;
 }
 
+// Resident blocks per SM of the context's kernel for this program set.
+static gtap_status kernel_occupancy(gtap_ctx* c, unsigned pset, size_t smem, int* occ) {
+    if (c->occ_blocks == 0 || c->occ_pset != pset || c->occ_smem != smem) {
+        int n = 0;
+        const cudaError_t e = (c->mode == GTAP_MODE_THREAD)
+                                  ? thread_kernel_occupancy(pset, c->cfg.scheduler, c->threads_per_block, smem, &n)
+                                  : block_kernel_occupancy(pset, c->threads_per_block, smem, &n);
+        if (e == cudaErrorInvalidValue) { cudaGetLastError(); return GTAP_ERR_INVALID_ARG; }   // no such instantiation
+        if (e != cudaSuccess) return GTAP_ERR_CUDA;
+        c->occ_pset = pset;
+        c->occ_smem = smem;
+        c->occ_blocks = n;
+    }
+    *occ = c->occ_blocks;
+    return GTAP_OK;
+}
+
 static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp, bool capturing, bool serving) {
     // inside a capture the kernel-timing events become event-record nodes of the graph
     auto record = [&](cudaEvent_t ev) {
@@ -644,11 +669,8 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
         P.warp_smem = (uint32_t)(thread_warp_smem(maxspawn) + thread_prog_smem(pset));
         smem = kThreadBlockSmem + (size_t)(c->threads_per_block / 32) * P.warp_smem;
         int occ = 0;
-        {
-            const cudaError_t oe = thread_kernel_occupancy(pset, c->cfg.scheduler, c->threads_per_block, smem, &occ);
-            if (oe == cudaErrorInvalidValue) { cudaGetLastError(); return GTAP_ERR_INVALID_ARG; }   // no such instantiation
-            if (oe != cudaSuccess) return GTAP_ERR_CUDA;
-        }
+        const gtap_status os = kernel_occupancy(c, pset, smem, &occ);
+        if (os != GTAP_OK) return os;
         if (occ < 1) return GTAP_ERR_INVALID_ARG;
         grid = std::min(c->grid, occ * c->sm_count);
         P.n_workers = (uint32_t)(grid * (c->threads_per_block / 32));
@@ -658,11 +680,8 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
         frame_bytes = block_record_bytes(pset, c->threads_per_block);
         smem = (size_t)block_rt_smem(maxspawn) + block_prog_smem(pset, c->threads_per_block);
         int occ = 0;
-        {
-            const cudaError_t oe = block_kernel_occupancy(pset, c->threads_per_block, smem, &occ);
-            if (oe == cudaErrorInvalidValue) { cudaGetLastError(); return GTAP_ERR_INVALID_ARG; }   // no such instantiation
-            if (oe != cudaSuccess) return GTAP_ERR_CUDA;
-        }
+        const gtap_status os = kernel_occupancy(c, pset, smem, &occ);
+        if (os != GTAP_OK) return os;
         if (occ < 1) return GTAP_ERR_INVALID_ARG;
         grid = std::min(c->grid, occ * c->sm_count);
         P.n_workers = (uint32_t)grid;
@@ -715,7 +734,7 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
             cudaSuccess)
             return GTAP_ERR_CUDA;
     }
-    if (launch_reset(P, 1, s) != cudaSuccess) return GTAP_ERR_CUDA;
+    if (launch_reset(P, 0, s) != cudaSuccess) return GTAP_ERR_CUDA;
     if (serving) {
         // the root table becomes a ring of request slots for the whole session
         P.serving = 1;
@@ -740,6 +759,7 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
         return GTAP_ERR_CUDA;
     }
     record(c->ev_k1);
+    if (launch_report(P, nroots, c->report_dev, c->roots_pinned_dev, s) != cudaSuccess) return GTAP_ERR_CUDA;
     lp->P = P;
     lp->pset = pset;
     lp->smem = smem;
@@ -765,50 +785,44 @@ gtap_status gtap_wait(gtap_ctx* c, uint64_t timeout_ms) {
             timed_out = true;
         }
         if (timed_out && (uint64_t)ms > timeout_ms + 10000ull) { return GTAP_ERR_TIMEOUT; }
-        std::this_thread::sleep_for(std::chrono::microseconds(ms < 2 ? 20 : 200));
+        // a short run is polled without a pause: the shortest sleep of the OS is about 70 us
+        if (ms >= 2) std::this_thread::sleep_for(std::chrono::microseconds(100));
     }
     c->running = false;
     float kms = 0.f, rms = 0.f;
     cudaEventElapsedTime(&kms, c->ev_k0, c->ev_k1);
-    cudaEventElapsedTime(&rms, c->ev_start, c->ev_stop);
-    cudaStream_t s = c->run_stream;
-    if (cudaMemcpyAsync(c->ctl_pinned, c->ctl, sizeof(DevControl), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(c->roots_pinned, c->roots, c->launched_roots * sizeof(RootEntry), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaMemcpyAsync(c->stats_pinned, c->stats, c->launched_workers * sizeof(WorkerStats), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return GTAP_ERR_CUDA;
+    cudaEventElapsedTime(&rms, c->ev_start, c->ev_k1);
     gtap_stats st{};
-    for (uint32_t w = 0; w < c->launched_workers; ++w) {
-        const WorkerStats& x = c->stats_pinned[w];
-        st.tasks_executed += x.tasks;
-        st.steps += x.steps;
-        st.pops += x.pops;
-        st.popped += x.popped;
-        st.steal_attempts += x.steal_attempts;
-        st.steals += x.steals;
-        st.stolen += x.stolen;
-        st.idle_iterations += x.idle;
-        st.pushes += x.pushes;
-        st.pushed += x.pushed;
-        st.tasks_created += x.spawned;
-        // thread mode: pop, steal, execute, retain/push, idle; block mode: acquire (pop or
-        // steal), -, body, post-step, idle
-        st.cycles_pop += x.pad[0]; st.cycles_steal += x.pad[1]; st.cycles_exec += x.pad[2];
-        st.cycles_push += x.pad[3]; st.cycles_idle += x.pad[4];
-    }
+    const RunReport& rep = *c->report;
+    const unsigned long long* x = rep.sums;
+    st.tasks_executed = x[kStTasks];
+    st.steps = x[kStSteps];
+    st.pops = x[kStPops];
+    st.popped = x[kStPopped];
+    st.steal_attempts = x[kStAttempts];
+    st.steals = x[kStSteals];
+    st.stolen = x[kStStolen];
+    st.idle_iterations = x[kStIdle];
+    st.pushes = x[kStPushes];
+    st.pushed = x[kStPushed];
+    st.tasks_created = x[kStSpawned];
+    // thread mode: pop, steal, execute, retain/push, idle; block mode: acquire (pop or
+    // steal), -, body, post-step, idle
+    st.cycles_pop = x[kStPop]; st.cycles_steal = x[kStSteal]; st.cycles_exec = x[kStExec];
+    st.cycles_push = x[kStPush]; st.cycles_idle = x[kStIdleCy];
     st.tasks_created += c->launched_roots;
-    st.frames_high_water = std::min<uint64_t>(c->ctl_pinned->bump.v, c->launched_frames);
-    st.scratch_used = c->ctl_pinned->scratch_top.v * kScratchBlock;
+    st.frames_high_water = std::min<uint64_t>(rep.bump, c->launched_frames);
+    st.scratch_used = rep.scratch_top * kScratchBlock;
     st.n_workers = (int)c->launched_workers;
     st.grid_blocks = c->launched_grid;
     st.threads_per_block = c->threads_per_block;
     st.kernel_ms = kms;
     st.run_ms = rms;
     c->last_stats = st;
-    c->last_err.code = c->ctl_pinned->err.code;
-    c->last_err.task_type = c->ctl_pinned->err.task_type;
-    c->last_err.worker = c->ctl_pinned->err.worker;
-    c->last_err.detail = c->ctl_pinned->err.detail;
+    c->last_err.code = rep.err.code;
+    c->last_err.task_type = rep.err.task_type;
+    c->last_err.worker = rep.err.worker;
+    c->last_err.detail = rep.err.detail;
     c->have_results = true;
     if (timed_out && c->last_err.code == 0) c->last_err.code = GTAP_ERR_TIMEOUT;
     return (gtap_status)c->last_err.code;

@@ -11,6 +11,7 @@
 
 #include "fmm_internal.h"
 #include "gtap.h"
+#include "launch.h"
 #include "scan.cuh"
 
 using namespace gtap;
@@ -183,6 +184,12 @@ struct gtap_fmm {
 };
 
 namespace {
+
+// Traversal constants (carried as a kernel argument: no staging copy) and cleared list counters.
+__global__ void k_dtt_begin(DttAux* aux, DttAux v, unsigned long long* counters) {
+    if (threadIdx.x == 0) *aux = v;
+    if (threadIdx.x < 4) counters[threadIdx.x] = 0;
+}
 
 float elapsed(cudaEvent_t a, cudaEvent_t b) {
     float ms = 0.f;
@@ -435,9 +442,10 @@ gtap_status gtap_fmm_traverse(gtap_fmm* f, gtap_ctx* ctx) {
         for (int d = 0; d < 3; ++d) cmax = std::max(cmax, std::max(std::fabs(f->box_h[d]), std::fabs(f->box_h[d] + f->box_h[3])));
         const double gap = std::ldexp(1.0, -50) * (cmax / f->box_h[3]) * std::ldexp(1.0, 21);
         ax.screen = gap < 1e-6 ? 1 : 0;
-        if (cudaMemcpyAsync(f->aux.p, &ax, sizeof(ax), cudaMemcpyHostToDevice, f->s) != cudaSuccess ||
-            cudaMemsetAsync(f->counters.p, 0, 4 * sizeof(unsigned long long), f->s) != cudaSuccess ||
-            cudaStreamSynchronize(f->s) != cudaSuccess)
+        k_dtt_begin<<<1, 32, 0, f->s>>>(f->aux.as<DttAux>(), ax, f->counters.as<unsigned long long>());
+        // the traversal runs on the context's stream, usually the plan's own
+        if (cudaGetLastError() != cudaSuccess ||
+            (ctx_stream(ctx) != f->s && cudaStreamSynchronize(f->s) != cudaSuccess))
             return GTAP_ERR_CUDA;
         if ((st = gtap_clear_roots(ctx)) != GTAP_OK) return st;
         gtap_fmm_dtt_args a{f, 0, 0};

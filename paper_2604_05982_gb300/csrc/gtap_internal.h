@@ -116,6 +116,18 @@ struct DevControl {
     Line128 admitted;          // serving: requests admitted so far
     Line128 gq_enq, gq_deq, gq_avail;   // central-queue scheduler: tickets and completed publications
     alignas(128) ErrorRecord err;
+    // end-of-run report: sums of the workers' counters (zeroed by the reset), blocks done, and how many
+    // slots of the chunk queue and the scratch queues the run used (the next reset re-arms only these)
+    alignas(128) unsigned long long sums[16];
+    unsigned int report_done, used_known;
+    unsigned long long cq_used, sq_used, lq_used;
+};
+
+// What a run leaves for the host, written to mapped host memory by the report kernel.
+struct RunReport {
+    unsigned long long sums[16];
+    unsigned long long bump, scratch_top;
+    ErrorRecord err;
 };
 
 // Serving: a root slot whose `done` word holds this value is free for a new request.

@@ -24,8 +24,14 @@ int block_kernel_maxspawn(unsigned pset, int bs);
 size_t block_prog_smem(unsigned pset, int bs);
 uint32_t block_record_bytes(unsigned pset, int bs);
 
-// Re-zero deques, pool, control words; write root records and push them.
-cudaError_t launch_reset(const KParams& P, int init_chunk_queue, cudaStream_t s);
+// Re-zero deques, pool, control words; write root records and push them.  init_queues 1: arm every slot of
+// the chunk and scratch queues; 0: only those that the last run used (launch_report has recorded them).
+cudaError_t launch_reset(const KParams& P, int init_queues, cudaStream_t s);
+// Sum the workers' counters and write the run's report and root results to mapped host memory.
+cudaError_t launch_report(const KParams& P, uint32_t n_roots, RunReport* report, RootEntry* roots, cudaStream_t s);
+
+// The stream a context's runs are ordered on (gtap_config.stream).
+cudaStream_t ctx_stream(const gtap_ctx* c);
 
 }  // namespace gtap
 

@@ -6,17 +6,22 @@
 
 namespace gtap {
 
-__global__ void reset_kernel(KParams P, int init_cq) {
+__global__ void reset_kernel(KParams P, int init_queues) {
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nth = (size_t)gridDim.x * blockDim.x;
     const uint32_t Q = P.n_queues;
     const uint32_t cap = P.ring_mask + 1;
-    if (init_cq)
-        for (size_t i = tid; i <= P.ncq_mask; i += nth) P.cq_seq[i] = i;
-    if (P.sq_seq != nullptr)
-        for (size_t i = tid; i <= P.sq_mask; i += nth) P.sq_seq[i] = i;
-    if (P.lq_seq != nullptr)
-        for (size_t i = tid; i <= P.lq_mask; i += nth) P.lq_seq[i] = i;
+    // a slot no ticket of the last run reached still holds its own index (megabytes of them for a 1 GiB pool)
+    const bool all = init_queues || P.ctl->used_known == 0;
+    auto rearm = [&](unsigned long long* seq, uint64_t mask, unsigned long long used) {
+        if (seq == nullptr) return;
+        const uint64_t n = all || used > mask ? mask + 1 : used;
+        for (size_t i = tid; i < n; i += nth) seq[i] = i;
+    };
+    rearm(P.cq_seq, P.ncq_mask, P.ctl->cq_used);
+    rearm(P.sq_seq, P.sq_mask, P.ctl->sq_used);
+    rearm(P.lq_seq, P.lq_mask, P.ctl->lq_used);
+    if (tid < 16) P.ctl->sums[tid] = 0;
     if (P.gq != nullptr) {
         // central queue: slot i holds root i (published: sequence i + 1), the rest are free (sequence i)
         for (size_t i = tid; i <= P.gq_mask; i += nth) {
@@ -80,6 +85,7 @@ __global__ void reset_kernel(KParams P, int init_cq) {
         P.ctl->gq_enq.v = P.gq ? P.n_roots : 0;
         P.ctl->gq_deq.v = 0;
         P.ctl->gq_avail.v = P.gq ? P.n_roots : 0;
+        P.ctl->report_done = 0;
         P.ctl->err.code = 0;
         P.ctl->err.task_type = -1;
         P.ctl->err.worker = -1;
@@ -87,8 +93,55 @@ __global__ void reset_kernel(KParams P, int init_cq) {
     }
 }
 
-cudaError_t launch_reset(const KParams& P, int init_cq, cudaStream_t s) {
-    reset_kernel<<<304, 256, 0, s>>>(P, init_cq);
+cudaError_t launch_reset(const KParams& P, int init_queues, cudaStream_t s) {
+    reset_kernel<<<304, 256, 0, s>>>(P, init_queues);
+    return cudaGetLastError();
+}
+
+// Thread t sums word t % 16 over every 16th worker row of its block's share; the
+// last block to finish writes the report.
+constexpr int kReportBlocks = 32, kReportThreads = 256;
+
+__global__ void __launch_bounds__(kReportThreads) report_kernel(KParams P, uint32_t n_roots, RunReport* report,
+                                                                RootEntry* roots) {
+    __shared__ unsigned long long sh[kReportThreads];
+    __shared__ bool last;
+    const int t = threadIdx.x;
+    const uint32_t rows = kReportThreads / 16;
+    const unsigned long long* st = reinterpret_cast<const unsigned long long*>(P.stats);
+    unsigned long long sum = 0;
+    for (uint32_t w = blockIdx.x * rows + t / 16; w < P.n_workers; w += gridDim.x * rows) sum += st[(size_t)w * 16 + t % 16];
+    sh[t] = sum;
+    // root results, 16 bytes a thread
+    const uint4* src = reinterpret_cast<const uint4*>(P.roots);
+    for (uint32_t i = blockIdx.x * kReportThreads + t; i < 2 * n_roots; i += gridDim.x * kReportThreads)
+        reinterpret_cast<uint4*>(roots)[i] = src[i];
+    __syncthreads();
+    if (t < 16) {
+        for (uint32_t k = 1; k < rows; ++k) sum += sh[t + 16 * k];
+        atomicAdd(&P.ctl->sums[t], sum);
+        __threadfence();
+    }
+    __syncthreads();
+    if (t == 0) last = atomicAdd(&P.ctl->report_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (t < 16) report->sums[t] = ld_cg64(&P.ctl->sums[t]);
+    if (t == 0) {
+        report->bump = P.ctl->bump.v;
+        report->scratch_top = P.ctl->scratch_top.v;
+        report->err = P.ctl->err;
+        P.ctl->cq_used = max(P.ctl->cq_enq.v, P.ctl->cq_deq.v);
+        P.ctl->sq_used = max(P.ctl->sc_enq.v, P.ctl->sc_deq.v);
+        P.ctl->lq_used = max(P.ctl->lc_enq.v, P.ctl->lc_deq.v);
+        P.ctl->used_known = 1;
+    }
+}
+
+cudaError_t launch_report(const KParams& P, uint32_t n_roots, RunReport* report, RootEntry* roots, cudaStream_t s) {
+    static_assert(sizeof(WorkerStats) == 128 && sizeof(RootEntry) == 32, "the report reads 16 words a worker and 2 x 16 bytes a root");
+    report_kernel<<<kReportBlocks, kReportThreads, 0, s>>>(P, n_roots, report, roots);
     return cudaGetLastError();
 }
 
