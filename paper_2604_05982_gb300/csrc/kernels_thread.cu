@@ -57,10 +57,11 @@ struct ThreadDispatch {
 // Resident 256-thread blocks per SM each program set is compiled for (the
 // register budget follows): k-clique tasks wait on L2 round trips, so it keeps
 // 4 blocks (64 registers); N-Queens and the full set measured faster with 80
-// registers at 3 blocks than capped at 64.
+// registers at 3 blocks than capped at 64; the Cilksort leaves hold 64 keys in
+// registers (2 blocks).
 template <unsigned PSET>
 constexpr int thread_min_blocks() {
-    return (PSET == PS_NQUEENS || PSET == PS_THREAD_ALL) ? 3 : 4;
+    return PSET == PS_CILKSORT ? 2 : (PSET == PS_NQUEENS || PSET == PS_THREAD_ALL) ? 3 : 4;
 }
 
 template <unsigned PSET, int SCHED>

@@ -3,6 +3,7 @@
 #pragma once
 #include "gtap_device.cuh"
 #include "programs_thread.cuh"
+#include "sort_networks.cuh"
 
 namespace gtap {
 
@@ -106,28 +107,6 @@ __device__ __forceinline__ void smem_window(const uint32_t* s, int base, int val
     }
 }
 
-// The N smallest of two ascending sequences a and b, ascending, into a.  The
-// element-wise minimum of a and reversed b holds exactly the N smallest of the
-// 2N keys and is bitonic (Batcher's bitonic merge, first half-cleaner); the
-// remaining half-cleaners sort it.  Only key values are produced, so which of
-// two equal keys is taken does not matter.
-template <int N>
-__device__ __forceinline__ void lowest_of_two_sorted(uint32_t (&a)[N], const uint32_t (&b)[N]) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) a[k] = min(a[k], b[N - 1 - k]);
-#pragma unroll
-    for (int j = N / 2; j > 0; j >>= 1) {
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            if ((k & j) == 0) {
-                const uint32_t x = a[k], y = a[k + j];
-                a[k] = min(x, y);
-                a[k + j] = max(x, y);
-            }
-        }
-    }
-}
-
 // The ITEMS outputs of merge-path position d of the runs A = s[a0, a0 + na)
 // and B = s[b0, b0 + nb) (padded indices), i of them taken from A: the lowest
 // ITEMS keys of the windows A[i, i + ITEMS) and B[d - i, d - i + ITEMS).
@@ -144,25 +123,6 @@ __device__ __forceinline__ void smem_window_merge(const uint32_t* s, int a0, int
 // registers with a bitonic network, then log2(BS) rounds of merging pairs of
 // sorted runs in shared memory, each thread producing kItems outputs of a
 // merge located by a merge-path search.
-template <int ITEMS>
-__device__ __forceinline__ void sort_registers(uint32_t (&x)[ITEMS]) {
-#pragma unroll
-    for (int k = 2; k <= ITEMS; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-#pragma unroll
-            for (int i = 0; i < ITEMS; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const uint32_t a = x[i], b = x[l];
-                    if ((a > b) == up) { x[i] = b; x[l] = a; }
-                }
-            }
-        }
-    }
-}
-
 template <int BS>
 __device__ void block_sort_leaf(const uint32_t* src, int n, uint32_t* dst, uint32_t* sh) {
     constexpr int kItems = kMsMaxLeaf / BS;
