@@ -352,16 +352,15 @@ typedef struct { const uint32_t* src; uint32_t* dst; uint32_t* tmp; uint64_t n; 
  * off/adj/src are the oriented DAG from gtap_kclique_orient (device, caller
  * owned, read only during the run).  Every DAG edge (u, v) of the root's
  * range (all edges: [0, m)) counts the
- * (k-2)-cliques of C = N+(u) n N+(v); a set larger than split_threshold
- * (<= 64, default 64) is materialised in the context's scratch arena
- * (gtap_config.scratch_bytes) and forked into child tasks over its branch
- * range; smaller ones are counted with 64-bit adjacency rows.  Where rows are
- * built (at least two more vertices to choose), the lanes of a warp that run
- * the same step process their edges or branches together, one at a time
- * (binary searches split over the lanes, C and its rows in the warp's shared
- * memory); elsewhere each lane intersects its own lists.  A first-level set is
- * written by its own task when that task starts (waiting first-level tasks
- * hold no scratch); deeper sets by the task that spawns them.
+ * (k-2)-cliques of C = N+(u) n N+(v).  A set of at most split_threshold
+ * (<= 64, default 64) members is counted where it is found; a larger one is a
+ * child task, which forks over its branch range with the set in the context's
+ * scratch arena (gtap_config.scratch_bytes), unless one branch away from the
+ * end: such a set of up to 256 members is counted whole, without scratch.
+ * The intersections of a warp's tasks are served by all its lanes together,
+ * one edge, branch or set at a time.  A first-level set is written by its own
+ * task when that task starts (waiting first-level tasks hold no scratch);
+ * deeper sets by the task that spawns them.
  * route 1: queue = recursion depth mod n_queues.  k in [3, 16].  Result: uint64 count.
  *
  * algorithm 1 (GTAP_KCLIQUE_PIVOT) counts by pivoting instead (Sec. 6.4.2, the

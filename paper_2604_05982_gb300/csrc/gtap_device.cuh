@@ -789,11 +789,18 @@ struct BlockIdle {
 
 // ---------------------------------------------------------------------------
 // Thread-mode scheduler loop (Algorithm 1), one instance per warp.
-// Dispatch is a functor: Dispatch::run(TaskCtx&) executes one step.
+// Dispatch is a functor: Dispatch::run(TaskCtx&) executes one step; program sets with
+// warp requests begin it, serve the requests by the whole warp, and finish it.
 // The longest sleep of an idle warp between steal rounds is a configuration
 // field (default 512 ns): longer sleeps relieve L2 of idle probing (the hashed
 // tree gained 8 % at 4 us) but slow the spread of work at start-up (fib and
 // N-Queens lost 15-25 % at 4 us), so the autotuner picks it per program.
+
+
+// Tasks a warp holds at a time when the whole warp serves them one after another
+// (Dispatch::kWarpRequests): 32 of them would keep one warp busy for
+// milliseconds while others find nothing to steal.
+constexpr int kWarpBatch = 2;
 
 template <class Dispatch, int SCHED = SCHED_BATCHED>
 __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_warp) {
@@ -847,6 +854,10 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     const int fhigh = 32 * (int)P.maxspawn + 2 * kChunk;
     constexpr int kProbes = 16;  // victims probed in parallel per steal attempt (one lane each)
     bool token = false;          // warp-uniform: this warp holds its block's probe token
+    // Tasks the warp takes for one step (warp-uniform): a k-clique kernel holds few orientation
+    // tasks at a time; a kernel with other programs keeps whole batches.
+    constexpr bool kAdaptive = Dispatch::kFirstBatch < 32;
+    int cap_now = Dispatch::kFirstBatch;
     // Fill steals (the warp holds tasks but fewer than 32) back off after failures:
     // after k failed attempts in a row the next 2^k - 1 steps skip them (k <= 6).
     // A warp with no task at all always tries.  Warp-uniform.
@@ -860,6 +871,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     };
 
     for (uint32_t iter = 0;; ++iter) {
+        const int cap = kAdaptive ? cap_now : 32;
         if ((iter & 63u) == 0u) {
             int ab = 0;
             // the host's abort word is read by every 64th warp only, and not at the start: a
@@ -947,7 +959,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             // ---- PopBatch (Algorithm 2) from the own queue: the retained class, else the fullest (DAQ).
             // The owner keeps an upper bound of each count (thieves only lower it), so an empty
             // queue costs no memory access and the CAS starts from a good guess.
-            if (cnt < 32) {
+            if (cnt < cap) {
                 int q = cls;
                 if (cnt == 0 && Q > 1) {
                     int best = (lane < Q) ? ws.hint[lane] : -1, bq = lane;
@@ -964,7 +976,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                     if (lane == 0) {
                         int old = ws.hint[q];
                         for (int it = 0; it < 64 && old > 0; ++it) {
-                            const int want = min(32 - cnt, old);
+                            const int want = min(cap - cnt, old);
                             const int got = atom_cas_acq_i32(&myq[q].count, old, old - want);
                             if (got == old) { claim = want; old -= want; break; }
                             old = got;
@@ -1016,7 +1028,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         }
         // ---- StealBatch.  SelectVictimQueue probes kProbes random victims at once (one
         // lane each) and picks the fullest, so an idle warp finds work in one round trip.
-        bool want_steal = (P.steal_policy & GTAP_STEAL_EMPTY) ? (cnt == 0) : (cnt < 32);
+        bool want_steal = (P.steal_policy & GTAP_STEAL_EMPTY) ? (cnt == 0) : (cnt < cap);
         if constexpr (SCHED == SCHED_GLOBAL) want_steal = false;   // no per-warp deques to steal from
         const bool fill = cnt > 0;
         if (want_steal && fill && fill_wait > 0) {
@@ -1108,7 +1120,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                         if (atom_cas_acq_i32(&vq->lock, 0, 1) == 0) {  // try-lock: never wait on a thief
                             int old = best;
                             for (int it = 0; it < 64 && old > 0; ++it) {
-                                int want = min(32 - cnt, old);
+                                int want = min(cap - cnt, old);
                                 if (P.steal_policy & GTAP_STEAL_HALF) want = min(want, (old + 1) >> 1);
                                 const int got = atom_cas_acq_i32(&vq->count, old, old - want);
                                 if (got == old) { claim = want; break; }
@@ -1196,12 +1208,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         bool done = false;               // this lane's task completed in this step
         unsigned long long rv = 0;
         uint32_t rw0 = 0, rparent = 0, rw3 = 0;
-        if (lane < cnt) {
-            if (P.fstate != nullptr) dbg_exec_check(P, tid, src, wid);
-            TaskCtx c(P, ws, tid, wid);
-            c.iter = iter;
-            dbg_log(P, tid, 3, wid, iter, (unsigned)c.pc() | ((unsigned)src << 8));
-            Dispatch::run(c);
+        auto after_step = [&](const TaskCtx& c) {
             spawned = c.nspawned;
             done = c.freed_self;
             rv = c.rv;
@@ -1210,6 +1217,43 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             rw3 = c.h.w3;
             if (!c.freed_self) dbg_log(P, tid, 4, wid, iter, 0);
             if (!c.freed_self && !c.staged_self) dbg_transition(P, tid, 2u, 1u, DBG_EXEC_NOT_ALLOCATED, c.type(), wid);
+        };
+        if constexpr (Dispatch::kWarpRequests) {
+            // the lanes without a task read lane 0's record (and leave it alone): they serve requests
+            const uint32_t t0 = __shfl_sync(0xffffffffu, tid, 0);
+            TaskCtx c(P, ws, lane < cnt ? tid : t0, wid);
+            c.iter = iter;
+            const bool asker = lane < cnt && Dispatch::may_ask(c.type());
+            if (lane < cnt) {
+                if (P.fstate != nullptr) dbg_exec_check(P, tid, src, wid);
+                dbg_log(P, tid, 3, wid, iter, (unsigned)c.pc() | ((unsigned)src << 8));
+            }
+            if (__any_sync(0xffffffffu, asker)) {
+                typename Dispatch::Request q;
+                bool asks = false;
+                if (asker) asks = Dispatch::begin(c, q);
+                __syncwarp();
+                if (__any_sync(0xffffffffu, asks)) {
+                    Dispatch::serve(ws, q);
+                    if (asks) Dispatch::finish(c, q);
+                }
+                if constexpr (kAdaptive) {
+                    const bool small = asker && q.warp_task;
+                    cap_now = 2 * __popc(__ballot_sync(0xffffffffu, small)) >= cnt ? kWarpBatch : 32;
+                }
+            } else if constexpr (kAdaptive) {
+                cap_now = 32;
+            }
+            if (lane < cnt && !asker) Dispatch::run(c);
+            __syncwarp();
+            if (lane < cnt) after_step(c);
+        } else if (lane < cnt) {
+            if (P.fstate != nullptr) dbg_exec_check(P, tid, src, wid);
+            TaskCtx c(P, ws, tid, wid);
+            c.iter = iter;
+            dbg_log(P, tid, 3, wid, iter, (unsigned)c.pc() | ((unsigned)src << 8));
+            Dispatch::run(c);
+            after_step(c);
         }
         __syncwarp();
         const unsigned done_mask = __ballot_sync(0xffffffffu, done);
@@ -1251,7 +1295,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                 qstar = __shfl_sync(0xffffffffu, bq, 0);
                 nq_star = ws.cls_count[qstar];
             }
-            const int nkeep = min(32, nq_star);
+            const int nkeep = min(kAdaptive ? cap_now : 32, nq_star);
             // capacity check per destination queue: uses head/tail, not count (Sec. 5.1.3)
             int overflow = 0;
             if (lane < Q) {

@@ -1,4 +1,6 @@
 // Thread-mode persistent kernels, one instantiation per program set.
+#include <type_traits>
+
 #include "launch.h"
 #include "gtap_device.cuh"
 #include "programs_thread.cuh"
@@ -8,6 +10,26 @@ namespace gtap {
 
 template <unsigned PSET>
 struct ThreadDispatch {
+    // A step may leave a request that the whole warp serves before the lane finishes the step.
+    static constexpr bool kWarpRequests = (PSET & PS_KCLIQUE) != 0;
+    static constexpr int kFirstBatch = PSET == PS_KCLIQUE ? kWarpBatch : 32;   // below 32: the batch adapts to the tasks
+    struct NoRequest {};
+    using Request = typename std::conditional<kWarpRequests, KcReq, NoRequest>::type;
+    __device__ static void serve(const WarpSh& ws, Request& q) {
+        if constexpr (kWarpRequests) kc_warp_requests<PSET != PS_KCLIQUE>(*reinterpret_cast<KcArea*>(ws.prog), q);
+    }
+    __device__ static void finish(TaskCtx& c, Request& q) {
+        if constexpr (kWarpRequests) {
+            if (c.type() == T_KCLIQUE_ROOT) kclique_range_finish(c, q);
+            else kclique_set_finish(c, q);
+        }
+    }
+    __device__ static bool may_ask(int type) { return type == T_KCLIQUE_ROOT || type == T_KCLIQUE_SET; }
+    // The first part of such a step; false when that completed it.
+    __device__ static bool begin(TaskCtx& c, Request& q) {
+        if constexpr (kWarpRequests) return c.type() == T_KCLIQUE_ROOT ? kclique_range_begin(c, q) : kclique_set_begin(c, q);
+        return false;
+    }
     __device__ static void run(TaskCtx& c) {
         switch (c.type()) {
         case T_FIB:
@@ -24,12 +46,6 @@ struct ThreadDispatch {
             break;
         case T_INTEGRATE:
             if constexpr ((PSET & PS_INTEGRATE) != 0) { integrate_step(c); return; }
-            break;
-        case T_KCLIQUE_ROOT:
-            if constexpr ((PSET & PS_KCLIQUE) != 0) { kclique_range_step(c); return; }
-            break;
-        case T_KCLIQUE_SET:
-            if constexpr ((PSET & PS_KCLIQUE) != 0) { kclique_set_dispatch(c); return; }
             break;
         case T_KCLIQUE_PIV:
             if constexpr ((PSET & PS_KCLIQUE) != 0) { kclique_piv_step(c); return; }

@@ -233,8 +233,10 @@ namespace gtap {
 // k-clique counting by orientation (Sec. 6.4.2).  For a DAG edge (u, v),
 // C = N+(u) n N+(v); count(S, 1) = |S|, count(S, j) = sum over w in S of
 // count(S n N+(w), j - 1).  A set of at most `thr` (<= 64) vertices is counted
-// inside the lane with 64-bit adjacency bitsets; a larger one is forked over
-// its branch range (the paper's split on the spawn-time estimate |C|).
+// where it is found, by its pairs or its 64-bit adjacency rows; a larger one is a
+// task that forks over its branch range (the paper's split on the spawn-time
+// estimate |C|), or counts its pairs when they are all that is left (see the
+// warp-cooperative passes below).
 //
 // Sets of the first level, C = N+(u) n N+(v), are spawned unmaterialised:
 // the record names P = N+(u), the vertex w = v and |C|, and the child writes C
@@ -259,7 +261,7 @@ constexpr uint32_t kKcSetSlotAcc = 6, kKcSetLocal = 56;
 constexpr uint32_t kKcSetPtr = 24, kKcSetLenLo = 32, kKcSetHiOwn = 40;
 constexpr uint32_t kKcLazy = 2;
 constexpr int kKcFan = 8;          // children per split
-constexpr int kKcMaxThr = 64;      // in-lane sets use 64-bit bitsets
+constexpr int kKcMaxThr = 64;      // sets counted by 64-bit rows
 
 // The root environment is immutable during a batch run (read-only path, L1);
 // in a served session the poller writes root slots while the kernel runs, so
@@ -317,55 +319,22 @@ static __device__ int kc_intersect(const int* a, int na, LA la, const int* b, in
     return cnt;
 }
 
-static __device__ unsigned long long kc_count_rows(const unsigned long long* row, int ns, int j);
-
-// count(S, j) for |S| <= 64 inside one lane, with 64-bit adjacency bitsets.
-static __device__ unsigned long long kc_count_small(const int* S, int ns, int j, const int64_t* off, const int* adj) {
-    if (j == 1) return (unsigned long long)ns;
+// The j-cliques (j >= 2) of a set of ns <= 64 members that start at member `first`, from the
+// set's adjacency rows (bit b of row[a]: member b is an out-neighbour of member a).
+static __device__ unsigned long long kc_count_rows(const unsigned long long* row, int ns, int j, int first) {
     if (ns < j) return 0;
-    unsigned long long row[kKcMaxThr];
-    for (int a = 0; a < ns; ++a) {
-        // row[a] = members of S that are out-neighbours of S[a]
-        const long long b0 = (long long)__ldg(reinterpret_cast<const long long*>(off) + S[a]);
-        const int len = (int)((long long)__ldg(reinterpret_cast<const long long*>(off) + S[a] + 1) - b0);
-        const int* nb = adj + b0;
-        unsigned long long bits = 0;
-        if (len > 4 * ns) {
-            int lo = 0;
-            for (int b = 0; b < ns && lo < len; ++b) {
-                const int x = S[b];
-                int hi = len;
-                while (lo < hi) { const int mid = (lo + hi) >> 1; if (__ldg(nb + mid) < x) lo = mid + 1; else hi = mid; }
-                if (lo < len && __ldg(nb + lo) == x) { bits |= 1ull << b; ++lo; }
-            }
-        } else {
-            int i = 0, b = 0;
-            while (i < len && b < ns) {   // branch-free merge
-                const int x = __ldg(nb + i), y = S[b];
-                bits |= (x == y) ? (1ull << b) : 0ull;
-                i += (x <= y) ? 1 : 0;
-                b += (y <= x) ? 1 : 0;
-            }
-        }
-        row[a] = bits;
-    }
-    return kc_count_rows(row, ns, j);
-}
-
-// count(S, j) from S's adjacency rows (bit b of row[a]: S[b] is an out-neighbour of S[a]), ns <= 64.
-static __device__ unsigned long long kc_count_rows(const unsigned long long* row, int ns, int j) {
-    if (j == 1) return (unsigned long long)ns;
-    if (ns < j) return 0;
-    const unsigned long long full = (ns == 64) ? ~0ull : ((1ull << ns) - 1ull);
-    if (j == 2) {
+    const unsigned long long m0 = row[first];
+    if (j == 2) return (unsigned)__popcll(m0);
+    if (j == 3) {
         unsigned long long t = 0;
-        for (int a = 0; a < ns; ++a) t += (unsigned)__popcll(row[a]);
+        for (unsigned long long w = m0; w; w &= w - 1) t += (unsigned)__popcll(m0 & row[__ffsll((long long)w) - 1]);
         return t;
     }
     // depth-first over choices; M = candidates at a level, R = those not yet tried there
     unsigned long long M[16], R[16];
-    M[0] = full;
-    R[0] = full;
+    if (__popcll(m0) < j - 1) return 0;
+    M[0] = m0;
+    R[0] = m0;
     int l = 0;
     unsigned long long total = 0;
     while (l >= 0) {
@@ -373,10 +342,8 @@ static __device__ unsigned long long kc_count_rows(const unsigned long long* row
         const int a = __ffsll((long long)R[l]) - 1;
         R[l] &= R[l] - 1;
         const unsigned long long mn = M[l] & row[a];
-        const int rem = j - l - 1;
-        if (rem == 1) {
-            total += (unsigned)__popcll(mn);
-        } else if (rem == 2) {
+        const int rem = j - l - 2;   // still to choose after `first`, l others and a
+        if (rem == 2) {
             for (unsigned long long w = mn; w; w &= w - 1) total += (unsigned)__popcll(mn & row[__ffsll((long long)w) - 1]);
         } else if (__popcll(mn) >= rem) {
             ++l;
@@ -808,192 +775,294 @@ __device__ __forceinline__ int kc_index_of(const int* C, int n, int x) {
     return (lo < n && C[lo] == x) ? lo : -1;
 }
 
-// The lanes of `mask` that run a cooperative pass (see below) and their shared area.
-struct KcCoop {
-    unsigned mask, below;
-    int lane, nact, rank, leader;
-    int* cbuf;
-    unsigned long long* rows;
-    int* claim;
+// Warp-cooperative passes (orientation).  A step runs in three parts: each lane
+// begins its own task and, where the work is intersections, leaves a request;
+// all 32 lanes of the warp, with a task or without, then take the requests one
+// after another, together; each lane finishes its task (spawn, join, return).
+// Lanes with short and long adjacency lists no longer wait for each other, and
+// the lanes of a warp that holds few tasks, as at the start and the end of a run,
+// help with them instead of standing idle.
+//
+// Kinds of requests:
+//   kKcEdges     DAG edges [lo, hi): per edge C = N+(u) n N+(v)
+//   kKcBranches  branches [lo, hi) of a set S (len members, in scratch): per branch C = S n N+(w)
+//   kKcPairs     a set of at most kKcSetMax members with one more vertex to choose after each
+//                branch: the DAG edges inside it.  The set is S in scratch, or (lazy) A n B,
+//                which is then never written to memory.
+// For edges and branches a C of at most `thr` members is counted (its pairs when need == 2,
+// from the 64-bit rows of the subgraph it induces when more); a larger one goes back to the
+// owner lane (di / dc, at most hi - lo of them), which spawns it.  (The last sets below a
+// branch, need == 2, are counted up to kKcSetMax members: written to scratch and queued, their
+// number outgrew the arena at k = 5, scale 20.)
+// Lanes of one warp may run tasks of different roots (batched or served graphs), so every
+// request carries its graph.
+//
+// Counting the pairs of a set needs no rows: a hit is counted when a member's out-neighbour is
+// found in the set, which is searched in shared memory.  (Per-lane merges of
+// a set's branches, two branches a task, left the lanes waiting for one L2 load after another,
+// in 57 tasks for a set of 92 members.)  Orientation and the 4-clique count of an R-MAT graph of
+// scale 17: 31.8 -> 11.8 ms; 400 served requests, a quarter of them such counts at scales
+// 10..14: 90 -> 65 ms.  Bound by issue: about 30 instructions for each list element searched.
+constexpr int kKcEdges = 1, kKcBranches = 2, kKcPairs = 3;
+constexpr int kKcSetMax = 256;
+// Per-warp area: the set, then the rows of a small set or 32 members' lists.
+struct KcArea {
+    int set[kKcSetMax];
+    union {
+        unsigned long long rows[kKcMaxThr];
+        struct {
+            const int* ptr[33];
+            int len[33];
+        } m;
+    };
+};
+constexpr int kKcCoopSmem = (int)((sizeof(KcArea) + 15) / 16 * 16);
+
+static_assert(kKcSetMax == 256, "kc_warp_pairs selects searches of up to 2 * 128 members");
+
+struct KcReq {
+    int kind = 0;
+    int need = 0, thr = 0;
+    uint32_t lo = 0, hi = 0, len = 0, own = 0;
+    const int* set = nullptr;            // S in scratch, or the list A of a lazy set
+    const int* list = nullptr;           // lazy set: the list B
+    int nlist = 0;
+    const long long* off = nullptr;
+    const int* adj = nullptr;
+    const int* src = nullptr;
+    bool warp_task = false;              // a task of this kind is served by the warp: hold few at a time
+    unsigned long long local = 0;        // the owner's count
+    int nd = 0;                          // sets too large to count here: item and size
+    uint32_t di[kKcFan];
+    int dc[kKcFan];
 };
 
-// Claims the warp's area for the lanes now converged here; false when another
-// group of the same warp holds it.
-__device__ __forceinline__ bool kc_coop_begin(KcCoop& k, int* area) {
-    k.mask = __activemask();
-    k.lane = threadIdx.x & 31;
-    k.below = (1u << k.lane) - 1u;
-    k.nact = __popc(k.mask);
-    k.rank = __popc(k.mask & k.below);
-    k.leader = __ffs((int)k.mask) - 1;
-    k.cbuf = area;
-    k.rows = reinterpret_cast<unsigned long long*>(area + kKcMaxThr);
-    k.claim = reinterpret_cast<int*>(k.rows + kKcMaxThr);
-    // the group's earlier writes (a set a lane has just materialised) become visible to all of it
-    __syncwarp(k.mask);
-    int got = 0;
-    if (k.lane == k.leader) got = atomicCAS(k.claim, 0, 1) == 0 ? 1 : 0;
-    return __shfl_sync(k.mask, got, k.leader) != 0;
-}
-__device__ __forceinline__ void kc_coop_end(const KcCoop& k) {
-    __syncwarp(k.mask);
-    if (k.lane == k.leader) atomicExch(k.claim, 0);
+__device__ __forceinline__ const int* kc_from(const void* p, int owner) {
+    return reinterpret_cast<const int*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(p), owner));
 }
 
-// C = S n L by the lanes of the group (S the shorter sorted list, split over the
-// lanes; L searched), kept in order in the area (up to kKcMaxThr members).
+// C = S n L by the warp (S the shorter sorted list, split over the lanes; L
+// searched where it is: a copy of it in shared memory measured slower), in order
+// in the area up to kKcSetMax members.  Returns |C|.
 template <bool SSET, bool LSET>
-__device__ __forceinline__ int kc_coop_collect(const KcCoop& k, const int* S, int ns, const int* L, int nl) {
+__device__ __forceinline__ int kc_warp_collect(KcArea& w, const int* S, int ns, const int* L, int nl) {
+    const int lane = threadIdx.x & 31;
     int cn = 0;
-    for (int b = 0; b < ns; b += k.nact) {
-        const int j = b + k.rank;
+    for (int b = 0; b < ns; b += 32) {
         int x = 0;
         bool in = false;
-        if (j < ns) {
-            x = kc_ld<SSET>(S + j);
+        if (b + lane < ns) {
+            x = kc_ld<SSET>(S + b + lane);
             in = kc_contains<LSET>(L, nl, x);
         }
-        const unsigned bal = __ballot_sync(k.mask, in);
-        if (in) {
-            const int p = cn + __popc(bal & k.below);
-            if (p < kKcMaxThr) k.cbuf[p] = x;   // C in ascending order (S is sorted, lanes in rank order)
-        }
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        const int p = cn + __popc(bal & lanemask_lt());
+        if (in && p < kKcSetMax) w.set[p] = x;   // ascending: S is sorted, lanes in order
         cn += __popc(bal);
     }
+    __syncwarp();
     return cn;
 }
-
-// One item, by all lanes of the group: C = A n B (sorted lists of the owner's
-// graph, B an out-list; A in the scratch arena when ASET, read through L2),
-// kept in order in the area; for need >= 2 and |C| <= thr also the rows of the
-// subgraph C induces, and the owner's count from them.  Returns |C|; *add gets
-// the owner's count (need == 1: |C|; 0 when C is larger than thr).
 template <bool ASET>
-__device__ __forceinline__ int kc_coop_item(const KcCoop& k, int owner, const int* A, int na, const int* B, int nb,
-                                            const long long* goff, const int* gadj, int need, int thr,
-                                            unsigned long long* add) {
-    const int cn = (na <= nb) ? kc_coop_collect<ASET, false>(k, A, na, B, nb)
-                              : kc_coop_collect<false, ASET>(k, B, nb, A, na);
-    __syncwarp(k.mask);
-    *add = 0;
-    if (need == 1) {
-        *add = (k.lane == owner) ? (unsigned long long)cn : 0ull;
-    } else if (cn >= need && cn <= thr) {
-        for (int a2 = 0; a2 < cn; ++a2) {
-            const int w = k.cbuf[a2];
-            const long long ow = __ldg(goff + w);
-            const int nw = (int)(__ldg(goff + w + 1) - ow);
+__device__ __forceinline__ int kc_warp_intersect(KcArea& w, const int* A, int na, const int* B, int nb) {
+    return (na <= nb) ? kc_warp_collect<ASET, false>(w, A, na, B, nb) : kc_warp_collect<false, ASET>(w, B, nb, A, na);
+}
+
+// The elements of m members' lists (w.m, closed by an endless one) as one sequence, lane l at
+// elements l, l + 32, ...; an element is loaded a round before it is searched in the set, which
+// is padded to 2 * HALF.  Returns this lane's hits.
+// HALF 0: the search is a loop over `half`.
+template <int HALF>
+__device__ __forceinline__ unsigned kc_pair_rounds(const KcArea& w, int m, int rounds, int half = HALF) {
+    const int lane = threadIdx.x & 31;
+    int r = 0, o = lane, ln = w.m.len[0];
+    const int* list = w.m.ptr[0];
+    auto next = [&] {   // the element at the lane's place, or -1 past the end
+        while (o >= ln) {
+            o -= ln;
+            ++r;
+            ln = w.m.len[r];
+            list = w.m.ptr[r];
+        }
+        const int x = r < m ? __ldg(list + o) : -1;
+        if (r < m) o += 32;
+        return x;
+    };
+    unsigned hits = 0;
+    int x = next();
+    for (int i = 0; i < rounds; ++i) {
+        const int nx = next();
+        int p = 0;   // the first member not less than x
+        if constexpr (HALF == 0) {
+            for (int h = half; h > 0; h >>= 1)
+                if (w.set[p + h - 1] < x) p += h;
+        } else {
+#pragma unroll
+            for (int h = HALF; h > 0; h >>= 1)
+                if (w.set[p + h - 1] < x) p += h;
+        }
+        hits += w.set[p] == x ? 1u : 0u;
+        x = nx;
+    }
+    return hits;
+}
+
+// This lane's share of the DAG edges inside the set w.set[0, cn) that leave members [lo, hi).
+template <bool COMPACT>
+__device__ __forceinline__ unsigned kc_warp_pairs(KcArea& w, int cn, int lo, int hi, const long long* off, const int* adj) {
+    const int lane = threadIdx.x & 31;
+    const int half = cn > 1 ? 1 << (31 - __clz(cn - 1)) : 1;   // half the padded size (which is >= 2)
+    for (int i = cn + lane; i < 2 * half; i += 32) w.set[i] = 0x7FFFFFFF;
+    __syncwarp();
+    unsigned hits = 0;
+    for (int base = lo; base < hi; base += 32) {
+        // every lane prepares one member's list
+        const int m = min(32, hi - base);
+        int n = 0;
+        if (lane < m) {
+            const int v = w.set[base + lane];
+            const long long o = __ldg(off + v);
+            n = (int)(__ldg(off + v + 1) - o);
+            w.m.ptr[lane] = adj + o;
+            w.m.len[lane] = n;
+        }
+        if (lane == 0) { w.m.ptr[m] = adj; w.m.len[m] = 0x7FFFFFFF; }
+        const int rounds = ((int)__reduce_add_sync(0xffffffffu, (unsigned)n) + 31) / 32;
+        __syncwarp();
+        if constexpr (COMPACT) {
+            hits += kc_pair_rounds<0>(w, m, rounds, half);
+        } else {
+            switch (half) {
+            case 1: hits += kc_pair_rounds<1>(w, m, rounds); break;
+            case 2: hits += kc_pair_rounds<2>(w, m, rounds); break;
+            case 4: hits += kc_pair_rounds<4>(w, m, rounds); break;
+            case 8: hits += kc_pair_rounds<8>(w, m, rounds); break;
+            case 16: hits += kc_pair_rounds<16>(w, m, rounds); break;
+            case 32: hits += kc_pair_rounds<32>(w, m, rounds); break;
+            case 64: hits += kc_pair_rounds<64>(w, m, rounds); break;
+            default: hits += kc_pair_rounds<128>(w, m, rounds); break;
+            }
+        }
+        __syncwarp();
+    }
+    return hits;
+}
+
+// This lane's share of the cliques of `need` vertices (>= 3) in the set cbuf[0, cn), cn <= 64:
+// the warp builds the 64-bit rows, then a lane counts the cliques that start at its members.
+__device__ __forceinline__ unsigned long long kc_warp_rows(KcArea& w, int cn, int need, const long long* off,
+                                                           const int* adj) {
+    const int lane = threadIdx.x & 31;
+    const int* cbuf = w.set;
+    unsigned long long* rows = w.rows;
+    for (int base = 0; base < cn; base += 32) {
+        long long ptr = 0;
+        int n = 0;
+        if (base + lane < cn) {
+            const int v = cbuf[base + lane];
+            ptr = __ldg(off + v);
+            n = (int)(__ldg(off + v + 1) - ptr);
+        }
+        const int m = min(32, cn - base);
+        for (int r = 0; r < m; ++r) {
+            const int* list = adj + __shfl_sync(0xffffffffu, ptr, r);
+            const int ln = __shfl_sync(0xffffffffu, n, r);
             unsigned long long bits = 0;
-            for (int b = k.rank; b < nw; b += k.nact) {
-                const int idx = kc_index_of(k.cbuf, cn, __ldg(gadj + ow + b));
+            for (int b = lane; b < ln; b += 32) {
+                const int idx = kc_index_of(cbuf, cn, __ldg(list + b));
                 if (idx >= 0) bits |= 1ull << idx;
             }
-            const unsigned r0 = __reduce_or_sync(k.mask, (unsigned)bits);
-            const unsigned r1 = __reduce_or_sync(k.mask, (unsigned)(bits >> 32));
-            if (k.rank == 0) k.rows[a2] = ((unsigned long long)r1 << 32) | r0;
+            const unsigned r0 = __reduce_or_sync(0xffffffffu, (unsigned)bits);
+            const unsigned r1 = __reduce_or_sync(0xffffffffu, (unsigned)(bits >> 32));
+            if (lane == 0) rows[base + r] = ((unsigned long long)r1 << 32) | r0;
         }
-        __syncwarp(k.mask);
-        if (k.lane == owner) *add = kc_count_rows(k.rows, cn, need);
     }
-    __syncwarp(k.mask);   // the area is rewritten by the next item
-    return cn;
+    __syncwarp();
+    unsigned long long total = 0;
+    for (int a = lane; a < cn; a += 32) total += kc_count_rows(rows, cn, need, a);
+    __syncwarp();   // the rows are rewritten by the next item
+    return total;
 }
 
-// Warp-cooperative passes (orientation, where C's rows are built: at least two
-// vertices still to choose): the lanes of a warp that reach the same task step
-// take every such lane's items (DAG edges of a range step, branches of a set
-// step) one after another, all together, so that lanes with short and long
-// adjacency lists no longer wait for each other.  Per item the
-// shorter list's elements are split over the lanes and looked up by binary
-// search in the longer one; the rows of a small C are built the same way, one
-// member's out-list per round.  Items whose C exceeds split_threshold go back
-// to their owner lane (di / dc, at most hi - lo of them), which spawns them.
-// Lanes of one warp may run tasks of different roots (batched or served
-// graphs), so an item's graph, k and threshold are broadcast from its owner.
-// Per-warp area: C (kKcMaxThr ints), its rows (kKcMaxThr words), a claim word.
-constexpr int kKcCoopSmem = kKcMaxThr * 4 + kKcMaxThr * 8 + 16;
-
-__device__ __forceinline__ const int* kc_bcast_ptr(unsigned mask, const void* p, int owner) {
-    return reinterpret_cast<const int*>(__shfl_sync(mask, reinterpret_cast<unsigned long long>(p), owner));
-}
-
-// Range step: the DAG edges [lo, hi) of this lane.  Returns false, having done
-// nothing, when the warp's area is in use.
-static __device__ __noinline__ bool kc_coop_edges(const gtap_kclique_args& e, int* area, uint32_t lo, uint32_t hi,
-                                                  int need, int thr, uint32_t* di, int* dc, int* dn,
-                                                  unsigned long long* local) {
-    KcCoop k;
-    if (!kc_coop_begin(k, area)) return false;
-    unsigned long long mine = 0;
-    int nd = 0;
-    for (unsigned m = k.mask; m != 0u; m &= m - 1u) {
+// The requests of the warp's lanes, by all 32 lanes (converged).
+// COMPACT: one search loop for every set size, for kernels that hold other programs too.
+template <bool COMPACT>
+static __device__ __noinline__ void kc_warp_requests(KcArea& w, KcReq& q) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned m = __ballot_sync(0xffffffffu, q.kind != 0); m != 0u; m &= m - 1u) {
         const int owner = __ffs((int)m) - 1;
-        const uint32_t olo = __shfl_sync(k.mask, lo, owner), ohi = __shfl_sync(k.mask, hi, owner);
-        const long long* goff = reinterpret_cast<const long long*>(kc_bcast_ptr(k.mask, e.off, owner));
-        const int* gadj = kc_bcast_ptr(k.mask, e.adj, owner);
-        const int* gsrc = kc_bcast_ptr(k.mask, e.src, owner);
-        const int oneed = __shfl_sync(k.mask, need, owner), othr = __shfl_sync(k.mask, thr, owner);
-        for (uint32_t ei = olo; ei < ohi; ++ei) {
-            const int u = __ldg(gsrc + ei), v = __ldg(gadj + ei);
-            const long long ou = __ldg(goff + u), ov = __ldg(goff + v);
-            const int nu = (int)(__ldg(goff + u + 1) - ou), nv = (int)(__ldg(goff + v + 1) - ov);
-            unsigned long long add;
-            const int cn = kc_coop_item<false>(k, owner, gadj + ou, nu, gadj + ov, nv, goff, gadj, oneed, othr, &add);
-            mine += add;
-            if (k.lane == owner && oneed >= 2 && cn >= oneed && cn > othr) {
-                di[nd] = ei;
-                dc[nd] = cn;
-                ++nd;
+        const int kind = __shfl_sync(0xffffffffu, q.kind, owner);
+        const int need = __shfl_sync(0xffffffffu, q.need, owner), thr = __shfl_sync(0xffffffffu, q.thr, owner);
+        const uint32_t lo = __shfl_sync(0xffffffffu, q.lo, owner), hi = __shfl_sync(0xffffffffu, q.hi, owner);
+        const int len = (int)__shfl_sync(0xffffffffu, q.len, owner);
+        const int* set = kc_from(q.set, owner);
+        const long long* off = reinterpret_cast<const long long*>(kc_from(q.off, owner));
+        const int* adj = kc_from(q.adj, owner);
+        unsigned long long mine = 0;
+        if (kind == kKcPairs) {
+            const int* list = kc_from(q.list, owner);
+            int cn = len;
+            if (list != nullptr) {
+                cn = kc_warp_intersect<false>(w, set, len, list, __shfl_sync(0xffffffffu, q.nlist, owner));
+                mine = kc_warp_pairs<COMPACT>(w, cn, 0, cn, off, adj);
+            } else {
+                for (int i = lane; i < cn; i += 32) w.set[i] = __ldcg(set + i);
+                __syncwarp();
+                mine = kc_warp_pairs<COMPACT>(w, cn, (int)lo, (int)hi, off, adj);
             }
+        } else {
+            // at most kKcFan items: lane i prepares item lo + i
+            const int* src = kc_from(q.src, owner);
+            const int items = (int)(hi - lo);
+            long long oa = 0, ob = 0;
+            int na = len, nb = 0;
+            if (lane < items) {
+                int v;
+                if (kind == kKcEdges) {
+                    const int u = __ldg(src + lo + lane);
+                    v = __ldg(adj + lo + lane);
+                    oa = __ldg(off + u);
+                    na = (int)(__ldg(off + u + 1) - oa);
+                } else {
+                    v = __ldcg(set + lo + lane);
+                }
+                ob = __ldg(off + v);
+                nb = (int)(__ldg(off + v + 1) - ob);
+            }
+            int nd = 0;
+            for (int i = 0; i < items; ++i) {
+                const int ina = __shfl_sync(0xffffffffu, na, i), inb = __shfl_sync(0xffffffffu, nb, i);
+                const int* A = adj + __shfl_sync(0xffffffffu, oa, i);
+                const int* B = adj + __shfl_sync(0xffffffffu, ob, i);
+                const int cn = kind == kKcEdges ? kc_warp_intersect<false>(w, A, ina, B, inb)
+                                                : kc_warp_intersect<true>(w, set, ina, B, inb);
+                if (cn < need) continue;
+                if (cn > thr && (kind == kKcEdges || need != 2 || cn > kKcSetMax)) {
+                    if (lane == owner) { q.di[nd] = lo + (uint32_t)i; q.dc[nd] = cn; }
+                    ++nd;
+                } else if (need == 2) {
+                    mine += kc_warp_pairs<COMPACT>(w, cn, 0, cn, off, adj);
+                } else {
+                    mine += kc_warp_rows(w, cn, need, off, adj);
+                }
+            }
+            if (lane == owner) q.nd = nd;
         }
+        // the owner's count: the sum over the lanes
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+        if (lane == owner) q.local = mine;
+        __syncwarp();
     }
-    kc_coop_end(k);
-    *dn = nd;
-    *local = mine;
-    return true;
 }
 
-// Set step: the branches [lo, hi) of this lane's set (len members, in the
-// scratch arena).  Returns false, having done nothing, when the area is in use.
-static __device__ __noinline__ bool kc_coop_branches(const gtap_kclique_args& e, int* area, const int* set, uint32_t len,
-                                                     uint32_t lo, uint32_t hi, int need, int thr, uint32_t* di, int* dc,
-                                                     int* dn, unsigned long long* local) {
-    KcCoop k;
-    if (!kc_coop_begin(k, area)) return false;
-    unsigned long long mine = 0;
-    int nd = 0;
-    for (unsigned m = k.mask; m != 0u; m &= m - 1u) {
-        const int owner = __ffs((int)m) - 1;
-        const uint32_t olo = __shfl_sync(k.mask, lo, owner), ohi = __shfl_sync(k.mask, hi, owner);
-        const uint32_t olen = __shfl_sync(k.mask, len, owner);
-        const int* oset = kc_bcast_ptr(k.mask, set, owner);
-        const long long* goff = reinterpret_cast<const long long*>(kc_bcast_ptr(k.mask, e.off, owner));
-        const int* gadj = kc_bcast_ptr(k.mask, e.adj, owner);
-        const int oneed = __shfl_sync(k.mask, need, owner), othr = __shfl_sync(k.mask, thr, owner);
-        for (uint32_t i = olo; i < ohi; ++i) {
-            const int w = __ldcg(oset + i);
-            const long long ow = __ldg(goff + w);
-            const int nw = (int)(__ldg(goff + w + 1) - ow);
-            unsigned long long add;
-            const int cn = kc_coop_item<true>(k, owner, oset, (int)olen, gadj + ow, nw, goff, gadj, oneed, othr, &add);
-            mine += add;
-            if (k.lane == owner && oneed >= 2 && cn >= oneed && cn > othr) {
-                di[nd] = i;
-                dc[nd] = cn;
-                ++nd;
-            }
-        }
-    }
-    kc_coop_end(k);
-    *dn = nd;
-    *local = mine;
-    return true;
-}
-
-static __device__ void kclique_range_step(TaskCtx& c) {
+// First part of the range step: returns true with a request for the warp, or false when the
+// step is complete.
+static __device__ bool kclique_range_begin(TaskCtx& c, KcReq& q) {
     const KcRangeSpawn a = c.load<KcRangeSpawn>();
     const gtap_kclique_args& e = kc_env(c.P, a.root);
-    if (c.pc() != 0) { c.ret(a.acc + a.local); return; }
+    q.warp_task = e.algorithm != GTAP_KCLIQUE_PIVOT;
+    if (c.pc() != 0) { c.ret(a.acc + a.local); return false; }
     const uint32_t n = a.hi - a.lo;
     if (n > (uint32_t)kKcFan) {
         const uint32_t per = (n + kKcFan - 1) / kKcFan;
@@ -1001,85 +1070,104 @@ static __device__ void kclique_range_step(TaskCtx& c) {
             c.spawn(T_KCLIQUE_ROOT, kKcRangeSlotAcc, kc_queue(e, 0), KcRangeSpawn{a.root, s, min(a.hi, s + per), 0u, 0ull, 0ull},
                     kFlagAccumulate);
         c.join(1, kc_queue(e, 0));
-        return;
+        return false;
     }
     const int thr = e.split_threshold;
     const int need = e.k - 2;
     const bool pivot = e.algorithm == GTAP_KCLIQUE_PIVOT;
-    unsigned long long local = 0;
-    uint32_t dei[kKcFan];
-    int dcn[kKcFan];
-    int dn = 0;
-    if (!pivot && need >= 2 &&
-        kc_coop_edges(e, reinterpret_cast<int*>(c.ws.prog), a.lo, a.hi, need, thr, dei, dcn, &dn, &local)) {
-        // orientation, warp-cooperative pass done; the sets too large to count there become set tasks
-        for (int q = 0; q < dn; ++q) {
-            const uint32_t ei = dei[q];
-            const int u = __ldg(e.src + ei), v = __ldg(e.adj + ei);
-            const long long ou = kc_off(e, u);
-            const int nu = (int)(kc_off(e, u + 1) - ou);
-            c.spawn(T_KCLIQUE_SET, kKcRangeSlotAcc, kc_queue(e, 1),
-                    KcSetSpawn{a.root, (uint32_t)need, (unsigned long long)(e.adj + ou), (uint32_t)nu, (uint32_t)v,
-                               (uint32_t)dcn[q], kKcLazy, 0ull, 0ull},
-                    kFlagAccumulate);
-        }
-        if (c.nspawned == 0) { c.ret(local); return; }
-        st_cg64(c.frame + kKcRangeLocal, local);
-        c.join(1, kc_queue(e, 0));
-        return;
+    if (!pivot && need >= 2) {
+        q.kind = kKcEdges;
+        q.need = need;
+        q.thr = thr;
+        q.lo = a.lo;
+        q.hi = a.hi;
+        q.off = reinterpret_cast<const long long*>(e.off);
+        q.adj = e.adj;
+        q.src = e.src;
+        return true;
     }
+    unsigned long long local = 0;
     int C[kKcMaxThr];
     for (uint32_t ei = a.lo; ei < a.hi; ++ei) {
         const int u = __ldg(e.src + ei), v = __ldg(e.adj + ei);
         const long long ou = kc_off(e, u), ov = kc_off(e, v);
         const int nu = (int)(kc_off(e, u + 1) - ou), nv = (int)(kc_off(e, v + 1) - ov);
-        const int cn = kc_intersect(e.adj + ou, nu, AdjLoad{}, e.adj + ov, nv, AdjLoad{}, C, pivot ? kKcMaxThr : thr);
+        const int cn = kc_intersect(e.adj + ou, nu, AdjLoad{}, e.adj + ov, nv, AdjLoad{}, C, kKcMaxThr);
         if (need == 1) { local += (unsigned)cn; continue; }
         if (cn < need) continue;
+        // pivoting
         if (cn <= thr) {
-            local += pivot ? kp_count_small(C, cn, need, e.off, e.adj) : kc_count_small(C, cn, need, e.off, e.adj);
+            local += kp_count_small(C, cn, need, e.off, e.adj);
             continue;
         }
-        if (pivot && cn <= kKcMaxThr) {
-            if (!kp_spawn_split(c, e, a.root, C, cn, need, 1, kKcRangeSlotAcc)) return;
+        if (cn <= kKcMaxThr) {
+            if (!kp_spawn_split(c, e, a.root, C, cn, need, 1, kKcRangeSlotAcc)) return false;
             continue;
         }
-        if (pivot) {
-            // more than 64 members: a pivot node over multi-word bitsets, materialised when it runs
-            c.spawn(T_KCLIQUE_PIVB, kKcRangeSlotAcc, kc_queue(e, 1),
-                    KpbSpawn{a.root, (uint32_t)need | (kKpbLazy << 24), (unsigned long long)(e.adj + ou),
-                             (unsigned long long)(uint32_t)v | ((unsigned long long)(uint32_t)nu << 32),
-                             kpb_range((uint32_t)cn, (uint32_t)cn, 0, 1), 0ull, 0ull},
-                    kFlagAccumulate);
-            continue;
-        }
-        // the child materialises N+(u) n N+(v) when it runs and adds its count
-        // into this range task's accumulator
-        c.spawn(T_KCLIQUE_SET, kKcRangeSlotAcc, kc_queue(e, 1),
-                KcSetSpawn{a.root, (uint32_t)need, (unsigned long long)(e.adj + ou), (uint32_t)nu, (uint32_t)v, (uint32_t)cn,
-                           kKcLazy, 0ull, 0ull},
+        // more than 64 members: a pivot node over multi-word bitsets, materialised when it runs
+        c.spawn(T_KCLIQUE_PIVB, kKcRangeSlotAcc, kc_queue(e, 1),
+                KpbSpawn{a.root, (uint32_t)need | (kKpbLazy << 24), (unsigned long long)(e.adj + ou),
+                         (unsigned long long)(uint32_t)v | ((unsigned long long)(uint32_t)nu << 32),
+                         kpb_range((uint32_t)cn, (uint32_t)cn, 0, 1), 0ull, 0ull},
                 kFlagAccumulate);
     }
-    if (c.nspawned == 0) { c.ret(local); return; }
+    if (c.nspawned == 0) { c.ret(local); return false; }
     st_cg64(c.frame + kKcRangeLocal, local);
+    c.join(1, kc_queue(e, 0));
+    return false;
+}
+
+// Last part of the range step: the sets too large to count there become set tasks, which
+// materialise N+(u) n N+(v) when they run and add their count into this task's accumulator.
+static __device__ void kclique_range_finish(TaskCtx& c, const KcReq& q) {
+    const KcRangeSpawn a = c.load<KcRangeSpawn>();
+    const gtap_kclique_args& e = kc_env(c.P, a.root);
+    for (int i = 0; i < q.nd; ++i) {
+        const uint32_t ei = q.di[i];
+        const int u = __ldg(e.src + ei), v = __ldg(e.adj + ei);
+        const long long ou = kc_off(e, u);
+        const int nu = (int)(kc_off(e, u + 1) - ou);
+        c.spawn(T_KCLIQUE_SET, kKcRangeSlotAcc, kc_queue(e, 1),
+                KcSetSpawn{a.root, (uint32_t)q.need, (unsigned long long)(e.adj + ou), (uint32_t)nu, (uint32_t)v,
+                           (uint32_t)q.dc[i], kKcLazy, 0ull, 0ull},
+                kFlagAccumulate);
+    }
+    if (c.nspawned == 0) { c.ret(q.local); return; }
+    st_cg64(c.frame + kKcRangeLocal, q.local);
     c.join(1, kc_queue(e, 0));
 }
 
-// COOP: the warp-cooperative branch pass is compiled in (the dispatcher picks it
-// for orientation steps that build rows); without it the per-lane step keeps
-// the registers it had.
-template <bool COOP>
-static __device__ void kclique_set_step(TaskCtx& c) {
+static __device__ bool kclique_set_begin(TaskCtx& c, KcReq& q) {
     const KcSetSpawn a = c.load<KcSetSpawn>();
     const gtap_kclique_args& e = kc_env(c.P, a.root);
+    q.warp_task = e.algorithm != GTAP_KCLIQUE_PIVOT;
     if (c.pc() != 0) {
         // an owner frees its set once every task that reads it is done
         if (a.own == 1u) scratch_free(c.P, reinterpret_cast<const int*>(a.set), c.type(), c.worker);
         c.ret(a.acc + a.local);
-        return;
+        return false;
     }
     const int* set = reinterpret_cast<const int*>(a.set);
     uint32_t len = a.len, lo = a.lo, hi = a.hi, own = a.own;
+    const bool pivot = e.algorithm == GTAP_KCLIQUE_PIVOT;
+    const int need = (int)a.j - 1;
+    q.off = reinterpret_cast<const long long*>(e.off);
+    q.adj = e.adj;
+    if (!pivot && need == 1 && (own == kKcLazy ? hi : len) <= (uint32_t)kKcSetMax) {
+        q.kind = kKcPairs;
+        q.set = set;
+        q.len = len;
+        q.lo = lo;
+        q.hi = hi;
+        q.own = own;
+        if (own == kKcLazy) {
+            const int w = (int)a.lo;
+            const long long ow = kc_off(e, w);
+            q.list = e.adj + ow;
+            q.nlist = (int)(kc_off(e, w + 1) - ow);
+        }
+        return true;
+    }
     if (own == kKcLazy) {
         // materialise S = P n N+(w) (|S| = hi > thr, known from the spawn)
         const int w = (int)a.lo;
@@ -1087,7 +1175,7 @@ static __device__ void kclique_set_step(TaskCtx& c) {
         const int nw = (int)(kc_off(e, w + 1) - ow);
         bool pooled;
         int* S = kc_scratch_alloc(c, (int)a.hi, &pooled);
-        if (!S) return;
+        if (!S) return false;
         kc_intersect(set, (int)a.len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, S, (int)a.hi);
         set = S;
         len = a.hi;
@@ -1107,55 +1195,41 @@ static __device__ void kclique_set_step(TaskCtx& c) {
                     KcSetSpawn{a.root, a.j, (unsigned long long)set, len, s, min(hi, s + per), 0u, 0ull, 0ull},
                     kFlagAccumulate);
         c.join(1, kc_queue(e, depth));
-        return;
+        return false;
     }
     const int thr = e.split_threshold;
-    const int need = (int)a.j - 1;
-    const bool pivot = e.algorithm == GTAP_KCLIQUE_PIVOT;
-    unsigned long long local = 0;
-    uint32_t di[kKcFan];
-    int dc[kKcFan];
-    int dn = 0;
-    // cooperative only where C's rows are built (need >= 2): a count alone (need == 1) is one
-    // latency-bound search per branch, better overlapped across the lanes' own branches
-    if (COOP && !pivot && need >= 2 &&
-        kc_coop_branches(e, reinterpret_cast<int*>(c.ws.prog), set, len, lo, hi, need, thr, di, dc, &dn, &local)) {
-        // orientation, warp-cooperative pass done; this lane materialises and spawns its larger sets
-        for (int q = 0; q < dn; ++q) {
-            const int w = __ldcg(set + di[q]);
-            const long long ow = kc_off(e, w);
-            const int nw = (int)(kc_off(e, w + 1) - ow);
-            bool pooled;
-            int* S = kc_scratch_alloc(c, dc[q], &pooled);
-            if (!S) return;
-            kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, S, dc[q]);
-            c.spawn(T_KCLIQUE_SET, kKcSetSlotAcc, kc_queue(e, depth + 1),
-                    KcSetSpawn{a.root, (uint32_t)need, (unsigned long long)S, (uint32_t)dc[q], 0u, (uint32_t)dc[q],
-                               pooled ? 1u : 0u, 0ull, 0ull},
-                    kFlagAccumulate);
-        }
-        hi = lo;   // the per-lane loop below has nothing left to do
+    if (!pivot && need >= 2) {
+        q.kind = kKcBranches;
+        q.need = need;
+        q.thr = thr;
+        q.set = set;
+        q.len = len;
+        q.lo = lo;
+        q.hi = hi;
+        q.own = own;
+        return true;
     }
+    // a branch range of a set of more than kKcSetMax members (need == 1), or pivoting
+    unsigned long long local = 0;
     int C[kKcMaxThr];
     for (uint32_t i = lo; i < hi; ++i) {
         const int w = __ldcg(set + i);
         const long long ow = kc_off(e, w);
         const int nw = (int)(kc_off(e, w + 1) - ow);
-        const int cn = kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, C, pivot ? kKcMaxThr : thr);
+        const int cn = kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, C, kKcMaxThr);
         if (need == 1) { local += (unsigned)cn; continue; }
         if (cn < need) continue;
         if (cn <= thr) {
-            local += pivot ? kp_count_small(C, cn, need, e.off, e.adj) : kc_count_small(C, cn, need, e.off, e.adj);
+            local += kp_count_small(C, cn, need, e.off, e.adj);
             continue;
         }
-        if (pivot && cn <= kKcMaxThr) {
-            if (!kp_spawn_split(c, e, a.root, C, cn, need, depth + 1, kKcSetSlotAcc)) return;
+        if (cn <= kKcMaxThr) {
+            if (!kp_spawn_split(c, e, a.root, C, cn, need, depth + 1, kKcSetSlotAcc)) return false;
             continue;
         }
-        // deeper sets are materialised here, by the spawning lane (see the header)
         bool pooled;
         int* S = kc_scratch_alloc(c, cn, &pooled);
-        if (!S) return;
+        if (!S) return false;
         kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, S, cn);
         c.spawn(T_KCLIQUE_SET, kKcSetSlotAcc, kc_queue(e, depth + 1),
                 KcSetSpawn{a.root, (uint32_t)need, (unsigned long long)S, (uint32_t)cn, 0u, (uint32_t)cn, pooled ? 1u : 0u,
@@ -1165,19 +1239,38 @@ static __device__ void kclique_set_step(TaskCtx& c) {
     if (c.nspawned == 0) {
         if (own == 1u) scratch_free(c.P, set, c.type(), c.worker);
         c.ret(local);
-        return;
+        return false;
     }
     st_cg64(c.frame + kKcSetLocal, local);
     c.join(1, kc_queue(e, depth));
+    return false;
 }
 
-// A set step whose branches still need at least two more vertices (j >= 3) runs
-// the cooperative pass (orientation only); the rest take the lean per-lane step.
-__device__ __forceinline__ void kclique_set_dispatch(TaskCtx& c) {
-    const unsigned long long w2 = c.word<2>();   // record bytes 16..23: root, j
-    const uint32_t j = (uint32_t)(w2 >> 32);
-    if (c.pc() == 0 && j >= 3 && kc_env(c.P, (uint32_t)w2).algorithm != GTAP_KCLIQUE_PIVOT) kclique_set_step<true>(c);
-    else kclique_set_step<false>(c);
+static __device__ void kclique_set_finish(TaskCtx& c, const KcReq& q) {
+    const KcSetSpawn a = c.load<KcSetSpawn>();
+    const gtap_kclique_args& e = kc_env(c.P, a.root);
+    const int depth = e.k - 2 - (int)a.j + 1;
+    // deeper sets are materialised here, by the spawning lane (see the header)
+    for (int i = 0; i < q.nd; ++i) {
+        const int w = __ldcg(q.set + q.di[i]);
+        const long long ow = kc_off(e, w);
+        const int nw = (int)(kc_off(e, w + 1) - ow);
+        bool pooled;
+        int* S = kc_scratch_alloc(c, q.dc[i], &pooled);
+        if (!S) return;
+        kc_intersect(q.set, (int)q.len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, S, q.dc[i]);
+        c.spawn(T_KCLIQUE_SET, kKcSetSlotAcc, kc_queue(e, depth + 1),
+                KcSetSpawn{a.root, (uint32_t)q.need, (unsigned long long)S, (uint32_t)q.dc[i], 0u, (uint32_t)q.dc[i],
+                           pooled ? 1u : 0u, 0ull, 0ull},
+                kFlagAccumulate);
+    }
+    if (c.nspawned == 0) {
+        if (q.own == 1u) scratch_free(c.P, q.set, c.type(), c.worker);
+        c.ret(q.local);
+        return;
+    }
+    st_cg64(c.frame + kKcSetLocal, q.local);
+    c.join(1, kc_queue(e, depth));
 }
 
 }  // namespace gtap
