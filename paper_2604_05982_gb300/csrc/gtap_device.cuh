@@ -1428,6 +1428,10 @@ __device__ __forceinline__ BlockSh carve_block(char* base, int step_max) {
     return b;
 }
 
+// bs.ctrl[4] of a task whose join is its last act, and that task's mark in the top bit of `pending`.
+constexpr int kJoinLast = -1;
+constexpr uint32_t kPendingLast = 0x80000000u;
+
 // Block-mode task context: all threads of the block run the same step.
 struct BTaskCtx {
     const KParams& P;
@@ -1473,6 +1477,12 @@ struct BTaskCtx {
     // Block-collective join (taskwait must be reached by all threads, Sec. 4.3).
     __device__ void join(int pc_next) {
         if (threadIdx.x == 0) bs.ctrl[4] = pc_next + 1;
+    }
+    // Join as the task's last act, for a task without a result: the last child completes this
+    // task too, and whoever that completes in turn, instead of scheduling a step that only returns
+    // (4 us a level of a merge tree's critical path).
+    __device__ void join_last() {
+        if (threadIdx.x == 0) bs.ctrl[4] = kJoinLast;
     }
     // Block-collective completion with per-thread return values: thread i of
     // the parent observes this task's thread i, and only on the thread that
@@ -1531,7 +1541,8 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
             uint32_t task = kNoTask;
             int state = 0;
             if (lane == 0) {
-                if ((iter & 15u) == 0u && abort_requested(P, (iter & 255u) == 0u)) {
+                // (the host's abort word is read by every 64th block, and not at the start)
+                if ((iter & 15u) == 0u && abort_requested(P, (bid & 63) == 0 && (iter & 127u) == 64u)) {
                     state = 2;
                 } else if (bs.misc[1] != kNoTask) {
                     task = bs.misc[1];   // the task retained from the previous step
@@ -1642,10 +1653,12 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                 int st = 0;
                 if (lane == 0) {
                     ++st_idle;
-                    if ((st_idle & 3ull) == 1ull) {
-                        if (ld_cg64(&P.ctl->roots_remaining.v) == 0ull) st = 2;
-                        else if (global_ns() > deadline) { raise_error(P, GTAP_ERR_TIMEOUT, -1, bid, P.timeout_ns); st = 2; }
-                        else if ((st_idle & 127ull) == 1ull && abort_requested(P, true)) st = 2;
+                    if (ld_cg64(&P.ctl->roots_remaining.v) == 0ull) st = 2;
+                    else if ((st_idle & 3ull) == 1ull && global_ns() > deadline) {
+                        raise_error(P, GTAP_ERR_TIMEOUT, -1, bid, P.timeout_ns);
+                        st = 2;
+                    } else if ((st_idle & 127ull) == 65ull && abort_requested(P, (bid & 63) == 0)) {
+                        st = 2;
                     }
                 }
                 state = __shfl_sync(0xffffffffu, st, 0);
@@ -1672,7 +1685,7 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                 backoff = 32;
             } else if (state == 0) {
                 if (lane == 0) __nanosleep(backoff);
-                backoff = min(backoff * 2, 1024);
+                backoff = min(backoff * 2, 256);
             }
             if (lane == 0) bs.ctrl[3] = state;
             __syncwarp();
@@ -1699,26 +1712,39 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                 char* f = frame_ptr(P, self);
                 const int jp = bs.ctrl[4];
                 st_spawned += (unsigned long long)bs.ctrl[2];
+                bool complete = bs.ctrl[5] != 0;
                 if (jp) {
                     // waiting-child count stored before any child is published
-                    int k = bs.ctrl[2];
-                    uint32_t w0 = (h.w0 & ~0xFF00u) | ((uint32_t)(jp - 1) << 8);
-                    __stcg(reinterpret_cast<uint2*>(f), make_uint2(w0, (uint32_t)k));
-                    if (k == 0) bs.staged_id[bs.ctrl[2]++] = self;
-                }
-                if (bs.ctrl[5]) {
-                    __threadfence();
-                    if (h.parent & kRootBit) {
-                        RootEntry* r = &P.roots[h.parent & ~kRootBit];
-                        atomicExch(&r->done, 1u);
-                        atomicAdd(&P.ctl->roots_remaining.v, ~0ull);
+                    const int k = bs.ctrl[2];
+                    if (jp == kJoinLast) {
+                        if (k == 0) complete = true;
+                        else __stcg(reinterpret_cast<uint2*>(f), make_uint2(h.w0, (uint32_t)k | kPendingLast));
                     } else {
-                        uint32_t old = atom_add_acqrel_u32(frame_ptr(P, h.parent) + 4, 0xFFFFFFFFu);
-                        if ((old & 0xFFFFFFu) == 1u) bs.staged_id[bs.ctrl[2]++] = h.parent;
+                        const uint32_t w0 = (h.w0 & ~0xFF00u) | ((uint32_t)(jp - 1) << 8);
+                        __stcg(reinterpret_cast<uint2*>(f), make_uint2(w0, (uint32_t)k));
+                        if (k == 0) bs.staged_id[bs.ctrl[2]++] = self;
                     }
-                    dbg_transition(P, self, 1u, 0u, DBG_DOUBLE_FREE, (int)(h.w0 & 0xFF), bid);
-                    int top = max(bs.ctrl[0], 0);
-                    if (top < bs.fcap) { bs.fstack[top] = self; bs.ctrl[0] = top + 1; }
+                }
+                if (complete) {
+                    __threadfence();
+                    uint32_t done = self, parent = h.parent;
+                    while (true) {
+                        dbg_transition(P, done, 1u, 0u, DBG_DOUBLE_FREE, (int)(h.w0 & 0xFF), bid);
+                        const int top = max(bs.ctrl[0], 0);
+                        if (top < bs.fcap) { bs.fstack[top] = done; bs.ctrl[0] = top + 1; }
+                        if (parent & kRootBit) {
+                            RootEntry* r = &P.roots[parent & ~kRootBit];
+                            atomicExch(&r->done, 1u);
+                            atomicAdd(&P.ctl->roots_remaining.v, ~0ull);
+                            break;
+                        }
+                        const uint32_t old = atom_add_acqrel_u32(frame_ptr(P, parent) + 4, 0xFFFFFFFFu);
+                        if ((old & 0xFFFFFFu) != 1u) break;
+                        if (!(old & kPendingLast)) { bs.staged_id[bs.ctrl[2]++] = parent; break; }
+                        // the parent's join was its last act: it is complete as well
+                        done = parent;
+                        parent = ld_cg32(frame_ptr(P, done) + 8);
+                    }
                 }
             }
             __syncwarp();

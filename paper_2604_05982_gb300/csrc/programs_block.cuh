@@ -33,10 +33,16 @@ __device__ __forceinline__ uint32_t* msort_buf(const gtap_mergesort_args& e, boo
 template <class Load>
 __device__ __forceinline__ unsigned long long merge_path(unsigned long long na, unsigned long long nb,
                                                          unsigned long long d, Load ld) {
+    // three candidates a step: half the dependent loads of a binary search
     unsigned long long lo = d > nb ? d - nb : 0, hi = d < na ? d : na;
     while (lo < hi) {
-        unsigned long long mid = (lo + hi) >> 1;
-        if (ld(true, mid) <= ld(false, d - 1 - mid)) lo = mid + 1; else hi = mid;
+        const unsigned long long q = (hi - lo) / 4, m1 = lo + q, m2 = lo + 2 * q, m3 = lo + 3 * q;
+        const bool t1 = ld(true, m1) <= ld(false, d - 1 - m1), t2 = ld(true, m2) <= ld(false, d - 1 - m2),
+                   t3 = ld(true, m3) <= ld(false, d - 1 - m3);
+        if (!t1) hi = m1;
+        else if (!t2) { lo = m1 + 1; hi = m2; }
+        else if (!t3) { lo = m2 + 1; hi = m3; }
+        else lo = m3 + 1;
     }
     return lo;
 }
@@ -169,9 +175,15 @@ __device__ void msort_fork_merge(BTaskCtx& c, const gtap_mergesort_args& e, uint
     const uint32_t* X = msort_buf(e, flags & 1u);
     const uint32_t* A = X + a_lo;
     const uint32_t* B = X + b_lo;
-    for (int p = threadIdx.x; p <= (int)pieces; p += BS) {
-        const unsigned long long d = total * (unsigned long long)p / pieces;
-        split[p] = merge_path(na, nb, d, [&](bool inA, unsigned long long k) { return __ldcg((inA ? A : B) + k); });
+    const auto key = [&](bool inA, unsigned long long k) { return __ldcg((inA ? A : B) + k); };
+    if ((int)pieces < BS / 8) {   // few boundaries: 8 lanes for each
+        const int p = (int)threadIdx.x / 8;
+        const unsigned long long d = total * (unsigned long long)min(p, (int)pieces) / pieces;
+        const unsigned long long sp = merge_path_group<8>(na, nb, d, key);
+        if (p <= (int)pieces && (threadIdx.x % 8) == 0) split[p] = sp;
+    } else {
+        for (int p = threadIdx.x; p <= (int)pieces; p += BS)
+            split[p] = merge_path(na, nb, total * (unsigned long long)p / pieces, key);
     }
     __syncthreads();
     if (threadIdx.x < (int)pieces) {
@@ -313,12 +325,12 @@ __device__ void msort_step(BTaskCtx& c) {
             c.ret_void();
         } else {
             msort_fork_merge<BS>(c, e, a.root, flags, a.lo, mid, mid, a.hi, a.lo);
-            c.join(2);
+            c.join_last();
         }
         return;
     }
     default:
-        c.ret_void();
+        break;
     }
 }
 
@@ -326,17 +338,13 @@ template <int BS>
 __device__ void mmerge_step(BTaskCtx& c) {
     const MmergeSpawn a = c.load<MmergeSpawn>();
     const gtap_mergesort_args& e = msort_env(c.P, a.root);
-    if (c.pc() == 0) {
-        const unsigned long long total = (a.a_hi - a.a_lo) + (a.b_hi - a.b_lo);
-        if (total <= e.merge_cutoff) {
-            msort_merge_piece<BS>(c, e, a.flags, a.a_lo, a.a_hi, a.b_lo, a.b_hi, a.out_lo);
-            c.ret_void();
-        } else {
-            msort_fork_merge<BS>(c, e, a.root, a.flags, a.a_lo, a.a_hi, a.b_lo, a.b_hi, a.out_lo);
-            c.join(1);
-        }
-    } else {
+    const unsigned long long total = (a.a_hi - a.a_lo) + (a.b_hi - a.b_lo);
+    if (total <= e.merge_cutoff) {
+        msort_merge_piece<BS>(c, e, a.flags, a.a_lo, a.a_hi, a.b_lo, a.b_hi, a.out_lo);
         c.ret_void();
+    } else {
+        msort_fork_merge<BS>(c, e, a.root, a.flags, a.a_lo, a.a_hi, a.b_lo, a.b_hi, a.out_lo);
+        c.join_last();
     }
 }
 
