@@ -487,8 +487,10 @@ __device__ __forceinline__ bool stage_task(const KParams& P, const WarpSh& ws, u
         return self_staged;
     }
     ws.staged_id[p] = id;
-    ws.staged_q[p] = (uint8_t)q;
-    if (P.n_queues > 1) atomicAdd(&ws.cls_count[q], 1);
+    if (P.n_queues > 1) {
+        ws.staged_q[p] = (uint8_t)q;
+        atomicAdd(&ws.cls_count[q], 1);
+    }
     return self_staged;
 }
 
@@ -802,6 +804,9 @@ struct BlockIdle {
 // milliseconds while others find nothing to steal.
 constexpr int kWarpBatch = 2;
 
+// Longest sleep of an idle warp that waits for its block's probe token.
+constexpr int kIdleWaitMax = 6400;
+
 template <class Dispatch, int SCHED = SCHED_BATCHED>
 __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_warp) {
     const int lane = threadIdx.x & 31;
@@ -850,6 +855,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     int cnt = 0;             // warp-uniform: lanes holding a task
     int cls = 0;             // warp-uniform: DAQ queue of the current batch
     int backoff = 32;
+    int wait_ns = 100;           // sleep of an idle warp without the probe token
     int ftop = 0;
     const int fhigh = 32 * (int)P.maxspawn + 2 * kChunk;
     constexpr int kProbes = 16;  // victims probed in parallel per steal attempt (one lane each)
@@ -1020,7 +1026,10 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             token = got == 1;
             if (!token) {
                 ++idle_n;
-                __nanosleep(200);
+                // up to 31 idle warps an SM: polling every 200 ns they took most of its issue
+                // slots from the one that works
+                __nanosleep(wait_ns);
+                wait_ns = min(wait_ns * 2, kIdleWaitMax);
                 phase(kStIdleCy);
                 continue;
             }
@@ -1196,6 +1205,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             continue;
         }
         backoff = 32;
+        wait_ns = 100;
 
         // ---- Ensure the free stack can serve every spawn of this step.
         ftop = pool_refill(P, ws.fstack, ftop, cnt * (int)P.maxspawn);
@@ -1325,11 +1335,28 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             }
             int kept = 0;
             int gbad = 0;
+            // One queue: the first staged tasks are kept, the others go to the ring in order, with no
+            // classes to rank.
+            if (Dispatch::kOneQueuePath && SCHED != SCHED_GLOBAL && Q == 1) {
+                for (int i = lane; i < nst; i += 32) {
+                    const uint32_t id = ws.staged_id[i];
+                    if (i < nkeep) {
+                        ws.retained[i] = id;
+                        dbg_log(P, id, 9, wid, iter, (unsigned)i);
+                    } else {
+                        const uint32_t pos = ws.tail[0] + (uint32_t)(i - nkeep);
+                        __stcg(&myring[pos & cap_mask], id);
+                        dbg_log(P, id, 6, wid, iter, pos & 0xFFFF);
+                    }
+                }
+                if (lane == 0) ws.push_off[0] = nst - nkeep;
+                __syncwarp();
+            } else
             for (int base = 0; base < nst; base += 32) {
                 const int i = base + lane;
                 const bool valid = i < nst;
                 uint32_t id = valid ? ws.staged_id[i] : kNoTask;
-                int q = valid ? (int)ws.staged_q[i] : 0;
+                int q = valid && Q > 1 ? (int)ws.staged_q[i] : 0;   // (written only with several queues)
                 const bool cand = valid && q == qstar;
                 const uint32_t km = __ballot_sync(0xffffffffu, cand);
                 const int rk = __popc(km & lanemask_lt());
