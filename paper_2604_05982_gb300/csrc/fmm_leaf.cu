@@ -306,7 +306,6 @@ __global__ void __launch_bounds__(kP2pBlock) k_p2p_fp64(EvalBufs e, const int4* 
     const bool target = i < count;
     const int ki = in.x + min(i, count - 1);
     const Dbl4 pt = e.pts[ki];
-    const double qi = target ? pt.w : 0.0;
     double acc = 0.0;
     if (own) {
         for (int k = slot; k < count; k += slots) {
@@ -334,8 +333,9 @@ __global__ void __launch_bounds__(kP2pBlock) k_p2p_fp64(EvalBufs e, const int4* 
             const Dbl4 p = e.pts[k];
             const double dx = pt.x - p.x, dy = pt.y - p.y, dz = pt.z - p.z;
             const double ir = rsqrt_fp64(fma(dz, dz, fma(dy, dy, dx * dx)));
-            acc = fma(valid ? p.w : 0.0, ir, acc);
-            mine = fma(qi, ir, mine);
+            // (selected, not weighted by zero: an infinite charge or 1/r stays where it belongs)
+            acc = valid ? fma(p.w, ir, acc) : acc;
+            mine = target ? fma(pt.w, ir, mine) : mine;
             if (gl == 0 && valid) atomicAdd(&near[k], mine);
             const double down = __shfl_down_sync(gmask, mine, 1, kGroup);
             mine = (gl == kGroup - 1 || pos + 1 < p0) ? 0.0 : down;
