@@ -189,7 +189,7 @@ def run_gpu(args):
     ms = ctx_for("mergesort", G.GTAP_MODE_BLOCK, 1, 256 << 20)
     t = ms.register("mergesort")
     ms.spawn(t, ms_args)
-    launches_per_step = 6   # each run: reset kernel + persistent scheduler kernel
+    launches_per_step = 9   # each run: reset kernel + persistent scheduler kernel + report kernel
 
     def step():
         t_nq = nq.run()
@@ -494,7 +494,7 @@ def _fmm_launches_per_instance(n_levels: int, mixed: bool) -> int:
     # bounding box, codes, 8 radix passes, refinement, gather, record check, leaf-local coordinates (mixed)
     tree = 2 + 8 + 1 + 1 + 1 + (1 if mixed else 0)
     upward = 1 + max(n_levels - 1, 0)
-    traverse = 2
+    traverse = 1 + 3   # list counters, then a run
     # two list groupings, multipole folding and M2L, L2L levels, near-field runs, P2P and L2P
     evaluate = 2 * 5 + 2 + max(n_levels - 1, 0) + 3
     return tree + upward + traverse + evaluate
@@ -825,7 +825,7 @@ def run_kclique(args):
                    if gold is not None else "sampled DAG-edge ranges equal the oracle's"),
         "e2e": {"value": ms, "unit": "ms/instance", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 16,
                 "note": "the edge list stays resident; the count is read back each step"},
-        "gpu_launches": (9 + 2) * args.steps,
+        "gpu_launches": (9 + 3) * args.steps,
         "clocks": clk.summary(),
     }
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
@@ -1037,7 +1037,7 @@ def run_serve(args):
                     "d2h_bytes_per_step": 48 * n_req,
                     "note": "the served rate is end to end: requests written by the host into the mapped inbox "
                             "(128 B each), completions read from the mapped outbox (48 B each)"},
-            "gpu_launches": 2,
+            "gpu_launches": 3,
             "waiting": {"inbox_mean": float(np.mean(backlog)), "inbox_max": int(max(backlog)),
                         "on_device_mean": float(np.mean(on_device)), "on_device_max": int(max(on_device)),
                         "samples": len(backlog),
@@ -1176,7 +1176,7 @@ def run_fib(args):
                 "h2d_bytes_per_step": 128, "d2h_bytes_per_step": 8,
                 "note": "root arguments in, result out through gtap_spawn_root / gtap_run / gtap_wait / "
                         "gtap_read_result (wall clock)"},
-        "gpu_launches": 2 * args.steps,
+        "gpu_launches": 3 * args.steps,
         "clocks": clk.summary(),
     }
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
@@ -1233,7 +1233,7 @@ def run_sched(args):
                                    "central queue vs non-batched vs batched stealing across grid sizes of "
                                    "256-thread blocks", "parallelism": "replicas"},
             "value_is": "batched stealing at 608 blocks (4 per SM)", "sweep": rows,
-            "gpu_launches": 2 * (1 + reps) * len(rows), "clocks": clk.summary()}
+            "gpu_launches": 3 * (1 + reps) * len(rows), "clocks": clk.summary()}
     _finish(line, world, rank)
 
 
@@ -1333,7 +1333,7 @@ def run_micro(args):
             "value_is": "thread mode, D = 25, compute_iters = 2048", **out,
             "thread_overtakes_block_at_depth": crossover("block_over_thread"),
             "thread_overtakes_block_cutoff_at_depth": crossover("cutoff_over_thread"),
-            "gpu_launches": 2 * (1 + reps) * (3 * 4 + 3 * 9 + 3 * 6), "clocks": clk.summary()}
+            "gpu_launches": 3 * (1 + reps) * (3 * 4 + 3 * 9 + 3 * 6), "clocks": clk.summary()}
     _finish(line, world, rank)
 
 
@@ -1432,7 +1432,7 @@ def run_batch(args):
             "e2e": {"value": BATCH_GRAPHS / t_graph, "unit": "instances/s", "h2d_bytes_per_step": 0,
                     "d2h_bytes_per_step": BATCH_GRAPHS * 32,
                     "note": "graphs resident on the device; each step reads the 64 counts back (gtap_wait)"},
-            "gpu_launches": 2 * (args.steps * 2 + args.steps // 2 * BATCH_GRAPHS),
+            "gpu_launches": 3 * (args.steps * 2 + args.steps // 2 * BATCH_GRAPHS),
             "clocks": clk.summary()}
     pc.close()
     c.close()
