@@ -356,7 +356,7 @@ typedef struct { const uint32_t* src; uint32_t* dst; uint32_t* tmp; uint64_t n; 
  * (<= 64, default 64) members is counted where it is found; a larger one is a
  * child task, which forks over its branch range with the set in the context's
  * scratch arena (gtap_config.scratch_bytes), unless one branch away from the
- * end: such a set of up to 256 members is counted whole, without scratch.
+ * end: such a set of up to 512 members is counted whole, without scratch.
  * The intersections of a warp's tasks are served by all its lanes together,
  * one edge, branch or set at a time.  A first-level set is written by its own
  * task when that task starts (waiting first-level tasks hold no scratch);

@@ -804,7 +804,9 @@ __device__ __forceinline__ int kc_index_of(const int* C, int n, int x) {
 // scale 17: 31.8 -> 11.8 ms; 400 served requests, a quarter of them such counts at scales
 // 10..14: 90 -> 65 ms.  Bound by issue: about 30 instructions for each list element searched.
 constexpr int kKcEdges = 1, kKcBranches = 2, kKcPairs = 3;
-constexpr int kKcSetMax = 256;
+// (the largest sets of an R-MAT graph of scale 20 hold between 256 and 512 members: its 4-clique
+// count takes 218 ms with 512 here, 364 ms with 256 and the rest by the per-lane path)
+constexpr int kKcSetMax = 512;
 // Per-warp area: the set, then the rows of a small set or 32 members' lists.
 struct KcArea {
     int set[kKcSetMax];
@@ -818,7 +820,7 @@ struct KcArea {
 };
 constexpr int kKcCoopSmem = (int)((sizeof(KcArea) + 15) / 16 * 16);
 
-static_assert(kKcSetMax == 256, "kc_warp_pairs selects searches of up to 2 * 128 members");
+static_assert(kKcSetMax == 512, "kc_warp_pairs selects searches of up to 2 * 256 members");
 
 struct KcReq {
     int kind = 0;
@@ -940,7 +942,8 @@ __device__ __forceinline__ unsigned kc_warp_pairs(KcArea& w, int cn, int lo, int
             case 16: hits += kc_pair_rounds<16>(w, m, rounds); break;
             case 32: hits += kc_pair_rounds<32>(w, m, rounds); break;
             case 64: hits += kc_pair_rounds<64>(w, m, rounds); break;
-            default: hits += kc_pair_rounds<128>(w, m, rounds); break;
+            case 128: hits += kc_pair_rounds<128>(w, m, rounds); break;
+            default: hits += kc_pair_rounds<256>(w, m, rounds); break;
             }
         }
         __syncwarp();

@@ -1,7 +1,7 @@
 """k-clique counts where the warp-served passes change path (GPU).
 
 Complete graphs have closed-form counts, C(n, k), and candidate sets of every size up to n - 2: around
-the row limit of 64, the powers of two of the search, and the 256 members a warp's set buffer holds.
+the row limit of 64, the powers of two of the search, and the 512 members a warp's set buffer holds.
 """
 import math
 
@@ -19,7 +19,7 @@ def _complete(n):
     return runner.DeviceGraph(n, np.stack([u, v], axis=1).astype(np.int32))
 
 
-@pytest.mark.parametrize("n,k", [(3, 3), (4, 4), (35, 4), (66, 4), (67, 4), (131, 4), (258, 4), (259, 4), (300, 4),
+@pytest.mark.parametrize("n,k", [(3, 3), (4, 4), (35, 4), (66, 4), (67, 4), (131, 4), (258, 4), (259, 4), (514, 4), (515, 4),
                                  (300, 3), (66, 5), (131, 5), (70, 6)])
 @pytest.mark.parametrize("thr,queues", [(64, 4), (2, 1)])
 def test_complete_graph_counts(n, k, thr, queues):
