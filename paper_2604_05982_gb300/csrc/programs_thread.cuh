@@ -664,6 +664,7 @@ static __device__ void kclique_pivb_step(TaskCtx& c) {
         for (int t = 0; t < W; ++t) {
             const int rem_bits = cn - t * 64;
             S[t] = rem_bits >= 64 ? ~0ull : ((1ull << rem_bits) - 1ull);
+            __stcg(setb + t, S[t]);   // read by the child tasks of a split branch range
         }
         // the set block lies inside the rows allocation: freeing the rows frees it (one free per block)
         flags = kKpbOwnRows | (kind == 1 ? kKpbRowsPooled : 0u) | (kind == 2 ? kKpbRowsLarge : 0u);
