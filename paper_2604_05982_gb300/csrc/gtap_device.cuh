@@ -860,10 +860,12 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     const int fhigh = 32 * (int)P.maxspawn + 2 * kChunk;
     constexpr int kProbes = 16;  // victims probed in parallel per steal attempt (one lane each)
     bool token = false;          // warp-uniform: this warp holds its block's probe token
-    // Tasks the warp takes for one step (warp-uniform): a k-clique kernel holds few orientation
-    // tasks at a time; a kernel with other programs keeps whole batches.
-    constexpr bool kAdaptive = Dispatch::kFirstBatch < 32;
-    int cap_now = Dispatch::kFirstBatch;
+    // Tasks the warp takes for one step (warp-uniform): a k-clique kernel holds few of the tasks that
+    // the warp serves, and whole batches of the others; so does its first claim, by the roots'
+    // kind (claims of two made the lane-served counts slow: triangles of an R-MAT graph of scale 16
+    // 3.14 ms with two always, 1.32 ms with 32).  A kernel with other programs keeps whole batches.
+    constexpr bool kAdaptive = Dispatch::kAdaptiveBatch;
+    int cap_now = kAdaptive && P.warp_roots ? kWarpBatch : 32;
     // Fill steals (the warp holds tasks but fewer than 32) back off after failures:
     // after k failed attempts in a row the next 2^k - 1 steps skip them (k <= 6).
     // A warp with no task at all always tries.  Warp-uniform.

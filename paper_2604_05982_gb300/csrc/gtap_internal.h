@@ -214,7 +214,7 @@ struct KParams {
     uint64_t seed;
     int steal_policy;
     int idle_backoff_ns;      // thread mode: longest sleep of an idle warp between steal rounds
-    int pad0;
+    int warp_roots;           // some root's tasks may be served by the whole warp (k-clique by orientation, k > 3)
     char* scratch;            // scratch blocks for programs (k-clique candidate sets), kScratchBlock bytes each
     uint64_t scratch_bytes;   // bytes of the block region
     unsigned long long* sq_seq;   // free-block queue: sequence numbers and block ids

@@ -17,7 +17,7 @@ struct ThreadDispatch {
     static constexpr bool kOneQueuePath = PSET == PS_UTS;
     // A step may leave a request that the whole warp serves before the lane finishes the step.
     static constexpr bool kWarpRequests = (PSET & PS_KCLIQUE) != 0;
-    static constexpr int kFirstBatch = PSET == PS_KCLIQUE ? kWarpBatch : 32;   // below 32: the batch adapts to the tasks
+    static constexpr bool kAdaptiveBatch = PSET == PS_KCLIQUE;   // the batch follows the tasks (kWarpBatch or 32)
     struct NoRequest {};
     using Request = typename std::conditional<kWarpRequests, KcReq, NoRequest>::type;
     __device__ static void serve(const WarpSh& ws, Request& q) {

@@ -1060,12 +1060,18 @@ static __device__ __noinline__ void kc_warp_requests(KcArea& w, KcReq& q) {
     }
 }
 
+// Whether a root's tasks ask the warp: orientation with at least two more vertices to choose after
+// an edge.  Pivoting and the triangle count run in their own lanes, 32 tasks a step.
+__device__ __forceinline__ bool kc_warp_root(const gtap_kclique_args& e) {
+    return e.algorithm != GTAP_KCLIQUE_PIVOT && e.k > 3;
+}
+
 // First part of the range step: returns true with a request for the warp, or false when the
 // step is complete.
 static __device__ bool kclique_range_begin(TaskCtx& c, KcReq& q) {
     const KcRangeSpawn a = c.load<KcRangeSpawn>();
     const gtap_kclique_args& e = kc_env(c.P, a.root);
-    q.warp_task = e.algorithm != GTAP_KCLIQUE_PIVOT;
+    q.warp_task = kc_warp_root(e);
     if (c.pc() != 0) { c.ret(a.acc + a.local); return false; }
     const uint32_t n = a.hi - a.lo;
     if (n > (uint32_t)kKcFan) {
@@ -1096,7 +1102,7 @@ static __device__ bool kclique_range_begin(TaskCtx& c, KcReq& q) {
         const int u = __ldg(e.src + ei), v = __ldg(e.adj + ei);
         const long long ou = kc_off(e, u), ov = kc_off(e, v);
         const int nu = (int)(kc_off(e, u + 1) - ou), nv = (int)(kc_off(e, v + 1) - ov);
-        const int cn = kc_intersect(e.adj + ou, nu, AdjLoad{}, e.adj + ov, nv, AdjLoad{}, C, kKcMaxThr);
+        const int cn = kc_intersect(e.adj + ou, nu, AdjLoad{}, e.adj + ov, nv, AdjLoad{}, need == 1 ? nullptr : C, kKcMaxThr);
         if (need == 1) { local += (unsigned)cn; continue; }
         if (cn < need) continue;
         // pivoting
@@ -1144,7 +1150,8 @@ static __device__ void kclique_range_finish(TaskCtx& c, const KcReq& q) {
 static __device__ bool kclique_set_begin(TaskCtx& c, KcReq& q) {
     const KcSetSpawn a = c.load<KcSetSpawn>();
     const gtap_kclique_args& e = kc_env(c.P, a.root);
-    q.warp_task = e.algorithm != GTAP_KCLIQUE_PIVOT;
+    // (branches of a set beyond kKcSetMax that need one more vertex are counted by their own lane)
+    q.warp_task = kc_warp_root(e) && (a.j > 2 || (a.own == kKcLazy ? a.hi : a.len) <= (uint32_t)kKcSetMax);
     if (c.pc() != 0) {
         // an owner frees its set once every task that reads it is done
         if (a.own == 1u) scratch_free(c.P, reinterpret_cast<const int*>(a.set), c.type(), c.worker);
@@ -1220,7 +1227,7 @@ static __device__ bool kclique_set_begin(TaskCtx& c, KcReq& q) {
         const int w = __ldcg(set + i);
         const long long ow = kc_off(e, w);
         const int nw = (int)(kc_off(e, w + 1) - ow);
-        const int cn = kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, C, kKcMaxThr);
+        const int cn = kc_intersect(set, (int)len, SetLoad{}, e.adj + ow, nw, AdjLoad{}, need == 1 ? nullptr : C, kKcMaxThr);
         if (need == 1) { local += (unsigned)cn; continue; }
         if (cn < need) continue;
         if (cn <= thr) {
