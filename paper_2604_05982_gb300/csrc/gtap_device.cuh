@@ -1017,14 +1017,21 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         phase(kStPop);
         // ---- Idle: wait for the block's probe token (not with the central queue, which has no victims).
         if (SCHED != SCHED_GLOBAL && cnt == 0 && !token) {
+            // The fullest class may have been stolen (its hint is now 0): the other own classes come
+            // first.  A warp that takes the token has no class left to pop, and only its own pushes
+            // raise a hint, so no warp works with the token that the block's others wait for.
             int got = 0;
             if (lane == 0) {
                 volatile BlockIdle* b = bidle;
+                int left = 0;
+                for (int k = 0; k < Q; ++k) left |= ws.hint[k];   // (never negative)
                 if (b->stop) got = 2;
+                else if (left != 0) got = 3;
                 else if (b->token == 0 && atomicCAS_block(&bidle->token, 0, 1) == 0) got = 1;
             }
             got = __shfl_sync(0xffffffffu, got, 0);
             if (got == 2) break;
+            if (got == 3) continue;
             token = got == 1;
             if (!token) {
                 ++idle_n;
