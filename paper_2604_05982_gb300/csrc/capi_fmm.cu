@@ -554,6 +554,15 @@ gtap_status gtap_fmm_copy_lists(const gtap_fmm* f, int32_t* m2l, int32_t* p2p) {
     return GTAP_OK;
 }
 
+gtap_status gtap_debug_fmm_gather(const double* pos, const double* q, const uint32_t* order, int64_t n, double* pts,
+                                  int32_t* flags) {
+    if (!pos || !q || !order || !pts || !flags || n < 1) return GTAP_ERR_INVALID_ARG;
+    if (launch_gather(pos, q, order, n, reinterpret_cast<Dbl4*>(pts), flags, nullptr) != cudaSuccess ||
+        cudaStreamSynchronize(nullptr) != cudaSuccess)
+        return GTAP_ERR_CUDA;
+    return GTAP_OK;
+}
+
 gtap_status gtap_fmm_destroy(gtap_fmm* f) {
     if (!f) return GTAP_ERR_INVALID_ARG;
     cudaStreamSynchronize(f->s);

@@ -149,6 +149,9 @@ size_t tree_work_bytes(long long n);
 // refinement of all levels; the gather of points into tree order, and the
 // structural check of the cell records (flags[1..3]).
 cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s);
+// Its gather of the points into tree order; sets flags[1] and skips a point whose index is not below n.
+cudaError_t launch_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags,
+                          cudaStream_t s);
 // Leaf-local FP32 coordinates (needs the cell count, known after the build).
 cudaError_t launch_leaf_local(const TreeBufs& b, int n_cells, cudaStream_t s);
 
@@ -192,3 +195,7 @@ gtap_status dtt_env(const gtap_fmm* plan, int target, int source, DttEnv* out);
 
 }  // namespace fmm
 }  // namespace gtap
+
+// Test entry: the gather on device arrays (pts: n x 4, flags: 4 words), synchronised.
+extern "C" gtap_status gtap_debug_fmm_gather(const double* pos, const double* q, const uint32_t* order, int64_t n,
+                                             double* pts, int32_t* flags);

@@ -30,6 +30,11 @@ namespace {
 
 constexpr int kRsBlock = 256;
 
+// A wait that runs out marks the build as failed.  The other waits of the build then end at once and the
+// kernels behind it do no work on keys that were never written: a failed build takes one wait's limit,
+// not one for each.
+__device__ __forceinline__ bool build_failed(const int* flags) { return *(const volatile int*)(flags + 1) != 0; }
+
 // Bounding cube: per-block min/max, and the last block to finish reduces those and
 // writes box = {lo x, lo y, lo z, side, scale} and the root cell.
 __global__ void __launch_bounds__(256) k_bbox(const double* pos, long long n, double* part, unsigned* done, double* box,
@@ -158,10 +163,15 @@ __global__ void __launch_bounds__(kRsBlock) k_rs_pass(const unsigned long long* 
     constexpr int kWarps = kRsBlock / 32;
     __shared__ unsigned cnt[kWarps][256];   // per warp: running digit counts, then the warp's first output position
     __shared__ unsigned tile_sh, wsum[kWarps];
+    __shared__ bool failed;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t == 0) tile_sh = atomicAdd(ticket, 1u);
+    if (t == 0) {
+        tile_sh = atomicAdd(ticket, 1u);
+        failed = build_failed(flags);
+    }
     for (int i = 0; i < kWarps; ++i) cnt[i][t] = 0;
     __syncthreads();
+    if (failed) return;
     const unsigned tile = tile_sh;
     const int shift = 8 * pass;
     const long long base = (long long)tile * (kRsBlock * ITEMS) + w * (32 * ITEMS) + lane;
@@ -209,25 +219,28 @@ __global__ void __launch_bounds__(kRsBlock) k_rs_pass(const unsigned long long* 
     unsigned first = incl - total;
     for (int i = 0; i < w; ++i) first += wsum[i];
     unsigned long long before = 0;
+    bool ok = true;
     if (tile > 0) {
-        bool ok = true;
         for (long long p = (long long)tile - 1; p >= 0 && ok; --p) {
             unsigned long long v = 0;
             int it = 0;
             do {
                 v = lb[(size_t)p * 256 + t];
                 ok = (v >> 48) == (tag >> 48);
-                if (!ok) __nanosleep(20);
+                if (!ok) {
+                    __nanosleep(20);
+                    if ((it & 255) == 255 && build_failed(flags)) break;
+                }
             } while (!ok && ++it < (1 << 20));
             before += v & kLbValue;
             if ((v >> 40 & 3ull) == 2ull) break;
         }
         if (!ok) flags[1] = 1;   // an earlier tile never reported: the build fails
-        lb[(size_t)tile * 256 + t] = tag | (2ull << 40) | ((before + own) & kLbValue);
+        else lb[(size_t)tile * 256 + t] = tag | (2ull << 40) | ((before + own) & kLbValue);
     }
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) cnt[i][t] += first + (unsigned)before;
-    __syncthreads();
+    if (__syncthreads_or(!ok)) return;
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
         const long long i = base + 32 * k;
@@ -252,6 +265,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, i
         met = 0;
         for (int it = 0; it < (1 << 22); ++it) {
             if (*(volatile unsigned*)count >= target) { met = 1; break; }
+            if ((it & 1023) == 1023 && build_failed(flags)) break;
             __nanosleep(32);
         }
         __threadfence();
@@ -288,6 +302,7 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
     __shared__ int red[kLvBlock / 32], total_sh, base_sh;
     const int t = threadIdx.x, lane = t & 31, o = t & 7, grp = t >> 3;
     const unsigned gshift = (unsigned)(lane & ~7);
+    if (build_failed(flags)) return;
     unsigned meet = 0;
     int l = 0;
     for (; l < kMaxLevel; ++l) {
@@ -399,9 +414,10 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
     }
 }
 
-__global__ void k_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts) {
+__global__ void k_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const uint32_t i = order[k];
+        if (i >= n) { flags[1] = 1; continue; }   // a sort that gave up leaves entries unwritten: any number
         pts[k] = make_dbl4(pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2], q[i]);
     }
 }
@@ -475,6 +491,12 @@ __global__ void k_check_tree(const int4* info, const int* lstart, int cap, long 
     }
 }
 
+cudaError_t launch_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags,
+                          cudaStream_t s) {
+    k_gather<<<grid_for(n, 256, 4096), 256, 0, s>>>(pos, q, order, n, pts, flags);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s) {
     const long long n = b.n;
     cudaError_t e = cudaMemsetAsync(b.work, 0, tree_work_bytes(n), s);
@@ -506,7 +528,7 @@ cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s) {
     // one block per SM, all resident (cooperative launch): the blocks wait for one another
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_levels), dim3(sms), dim3(kLvBlock), args, 0, s);
     if (e != cudaSuccess) return e;
-    k_gather<<<grid_for(n, 256, 4096), 256, 0, s>>>(b.pos, b.q, b.order, n, b.pts);
+    if ((e = launch_gather(b.pos, b.q, b.order, n, b.pts, b.flags, s)) != cudaSuccess) return e;
     k_check_tree<<<grid_for(b.cap_cells, 256, 1216), 256, 0, s>>>(b.info, b.lstart, b.cap_cells, n, b.flags);
     return cudaGetLastError();
 }
