@@ -222,6 +222,7 @@ EvalBufs eval_bufs(gtap_fmm* f, double* phi) {
     e.info = f->info.as<int4>();
     e.lat = f->lat.as<int4>();
     e.lat_unit = (float)(f->box_h[3] / 4194304.0);
+    e.close_unit = std::isfinite(f->box_h[5]) ? (float)(f->box_h[5] / (0.5 * f->box_h[3])) : INFINITY;
     e.lstart = f->lstart_h;
     e.pts = f->pts.as<Dbl4>();
     e.ploc = f->ploc.as<float4>();
@@ -557,10 +558,13 @@ gtap_status gtap_fmm_copy_lists(const gtap_fmm* f, int32_t* m2l, int32_t* p2p) {
 gtap_status gtap_debug_fmm_gather(const double* pos, const double* q, const uint32_t* order, int64_t n, double* pts,
                                   int32_t* flags) {
     if (!pos || !q || !order || !pts || !flags || n < 1) return GTAP_ERR_INVALID_ARG;
-    if (launch_gather(pos, q, order, n, reinterpret_cast<Dbl4*>(pts), flags, nullptr) != cudaSuccess ||
-        cudaStreamSynchronize(nullptr) != cudaSuccess)
-        return GTAP_ERR_CUDA;
-    return GTAP_OK;
+    DBuf box;
+    if (!box.ensure(8 * sizeof(double))) return GTAP_ERR_NO_MEMORY;
+    const bool ok = cudaMemset(box.p, 0, 8 * sizeof(double)) == cudaSuccess &&
+                    launch_gather(pos, q, order, n, reinterpret_cast<Dbl4*>(pts), flags, box.as<double>(), nullptr) == cudaSuccess &&
+                    cudaStreamSynchronize(nullptr) == cudaSuccess;
+    box.release();
+    return ok ? GTAP_OK : GTAP_ERR_CUDA;
 }
 
 gtap_status gtap_fmm_destroy(gtap_fmm* f) {

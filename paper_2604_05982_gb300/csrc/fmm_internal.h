@@ -124,7 +124,7 @@ struct TreeBufs {
     int leaf;
     const double* pos;            // input positions, n x 3 (device)
     const double* q;              // input charges (device)
-    double* box;                  // [8]: lo x/y/z, side, scale
+    double* box;                  // [8]: lo x/y/z, side, scale, largest |charge|
     double* bbox_part;            // [6 * kBoxParts]
     unsigned long long* keys[2];  // radix-sort ping-pong
     uint32_t* vals[2];
@@ -151,7 +151,7 @@ size_t tree_work_bytes(long long n);
 cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s);
 // Its gather of the points into tree order; sets flags[1] and skips a point whose index is not below n.
 cudaError_t launch_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags,
-                          cudaStream_t s);
+                          double* box, cudaStream_t s);
 // Leaf-local FP32 coordinates (needs the cell count, known after the build).
 cudaError_t launch_leaf_local(const TreeBufs& b, int n_cells, cudaStream_t s);
 
@@ -163,6 +163,7 @@ struct EvalBufs {
     const int4* info;
     const int4* lat;              // lattice centres (see TreeBufs)
     float lat_unit;               // side / 2^22: length of one lattice step
+    float close_unit;             // largest |charge| / root half side (see near_fp64 in fmm_leaf.cu)
     const int* lstart;            // host copy of the level starts
     const Dbl4* pts;
     const float4* ploc;

@@ -17,11 +17,39 @@ namespace fmm {
 namespace {
 
 // ---------------------------------------------------------------------------
+// Points much closer than their leaf's extent are not resolved by the mixed form's FP32 coordinates
+// relative to leaf centres: such a distance is off, or zero for distinct points, and the near sum
+// wrong, infinite or NaN.  The near sum of a target that one such pair dominates exceeds what well
+// separated points add up to (about half of q_max / h for each of them, h the leaf's half side);
+// it is taken again from the FP64 coordinates.  Below the limit a pair with the largest charge is more
+// than h / (kCloseSum + near points) apart, and its FP32 distance good to a few 1e-4.
+constexpr float kCloseSum = 1024.f;
+
+// The near sum of sorted point `own` of leaf c in FP64, by a warp.  (Points of one leaf at the same place do
+// not interact in the mixed form.)
+static __device__ __noinline__ double near_fp64(const EvalBufs& e, int c, int own) {
+    const int lane = threadIdx.x & 31;
+    const Dbl4 p = e.pts[own];
+    double sum = 0.0;
+    for (int j = e.p2p_off[c]; j < e.p2p_off[c + 1]; ++j) {
+        const int4 si = e.info[e.p2p_src[j]];
+        for (int k = si.x + lane; k < si.x + si.y; k += 32) {
+            const Dbl4 q = e.pts[k];
+            const double dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z, r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            if (r2 > 0.0) sum = fma(q.w, rsqrt(r2), sum);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    return sum;
+}
+
 // L2P: one block per leaf, one thread per point, nested Horner sums.
 constexpr int kL2pBlock = 64;
+static_assert(kL2pBlock >= kMaxLeaf, "one thread per point");
 
 template <class R>
-__global__ void __launch_bounds__(kL2pBlock) k_l2p(EvalBufs e, const double* near) {
+__global__ void __launch_bounds__(kL2pBlock, 32) k_l2p(EvalBufs e, const double* near) {
     __shared__ R lsm[n_coef(kMaxOrder)];
     const int c = blockIdx.x;
     const int4 in = e.info[c];
@@ -30,28 +58,39 @@ __global__ void __launch_bounds__(kL2pBlock) k_l2p(EvalBufs e, const double* nea
     for (int i = threadIdx.x; i < nt; i += kL2pBlock) lsm[i] = (R)e.L[(size_t)c * nt + i];
     __syncthreads();
     const Dbl4 g = e.geom[c];
-    for (int i = threadIdx.x; i < in.y; i += kL2pBlock) {
-        const int k = in.x + i;
-        R x, y, z;
-        if constexpr (sizeof(R) == 4) {
-            const float4 pl = e.ploc[k];
-            x = pl.x; y = pl.y; z = pl.z;
-        } else {
-            const Dbl4 pt = e.pts[k];
-            x = __dsub_rn(pt.x, g.x); y = __dsub_rn(pt.y, g.y); z = __dsub_rn(pt.z, g.z);
-        }
-        R sx = 0;
-        for (int a = p; a >= 0; --a) {
-            R sy = 0;
-            for (int b = p - a; b >= 0; --b) {
-                R sz = 0;
-                for (int cc = p - a - b; cc >= 0; --cc) sz = sz * z + lsm[cidx(a, b, cc)];
-                sy = sy * y + sz;
-            }
-            sx = sx * x + sy;
-        }
-        e.phi[e.order[k]] = near[k] + (double)sx;
+    const int i = threadIdx.x, k = in.x + min(i, in.y - 1);
+    if ((i & ~31) >= in.y) return;   // (a warp without a point; lanes past the last repeat it)
+    R x, y, z;
+    if constexpr (sizeof(R) == 4) {
+        const float4 pl = e.ploc[k];
+        x = pl.x; y = pl.y; z = pl.z;
+    } else {
+        const Dbl4 pt = e.pts[k];
+        x = __dsub_rn(pt.x, g.x); y = __dsub_rn(pt.y, g.y); z = __dsub_rn(pt.z, g.z);
     }
+    R sx = 0;
+    for (int a = p; a >= 0; --a) {
+        R sy = 0;
+        for (int b = p - a; b >= 0; --b) {
+            R sz = 0;
+            for (int cc = p - a - b; cc >= 0; --cc) sz = sz * z + lsm[cidx(a, b, cc)];
+            sy = sy * y + sz;
+        }
+        sx = sx * x + sy;
+    }
+    double nk = near[k];
+    if constexpr (sizeof(R) == 4) {
+        // the limit of a normal sum, compared by the double's high word
+        const int entries = e.p2p_off[c + 1] - e.p2p_off[c];
+        const float limit = (kCloseSum + (float)kMaxLeaf * (float)entries) * e.close_unit * (float)(1 << (in.w >> 8));
+        const unsigned limit_hi = (__float_as_uint(limit) >> 3) + (896u << 20);
+        for (unsigned m = __ballot_sync(0xffffffffu, ((unsigned)__double2hiint(nk) & 0x7FFFFFFFu) > limit_hi); m != 0u; m &= m - 1u) {
+            const int o = __ffs((int)m) - 1;
+            const double v = near_fp64(e, c, __shfl_sync(0xffffffffu, k, o));
+            if ((i & 31) == o) nk = v;
+        }
+    }
+    if (i < in.y) e.phi[e.order[k]] = nk + (double)sx;
 }
 
 // ---------------------------------------------------------------------------
@@ -87,7 +126,7 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-// 1/sqrt(x), the hardware approximation (inputs here are normal: distinct points)
+// 1/sqrt(x), the hardware approximation; infinite for zero and subnormal x (see near_fp64)
 __device__ __forceinline__ float rsqrt_ftz(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

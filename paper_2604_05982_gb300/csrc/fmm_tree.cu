@@ -36,7 +36,7 @@ constexpr int kRsBlock = 256;
 __device__ __forceinline__ bool build_failed(const int* flags) { return *(const volatile int*)(flags + 1) != 0; }
 
 // Bounding cube: per-block min/max, and the last block to finish reduces those and
-// writes box = {lo x, lo y, lo z, side, scale} and the root cell.
+// writes box = {lo x, lo y, lo z, side, scale, 0} and the root cell.
 __global__ void __launch_bounds__(256) k_bbox(const double* pos, long long n, double* part, unsigned* done, double* box,
                                               Dbl4* geom, int4* info, int4* lat, int* lstart, int* flags) {
     __shared__ double sh[6][256];
@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(256) k_bbox(const double* pos, long long n, do
     }
     box[3] = side;
     box[4] = __ddiv_rn(2097152.0, side);
+    box[5] = 0.0;   // largest |charge|: the gather's
     geom[0] = make_dbl4(c[0], c[1], c[2], half);
     info[0] = make_int4(0, (int)n, -1, 0);
     lat[0] = make_int4(1 << 21, 1 << 21, 1 << 21, 0);
@@ -414,12 +415,24 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
     }
 }
 
-__global__ void k_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags) {
+// (also the largest |charge| to 20 bits, in box[5]: the high words of non-negative doubles keep their order)
+__global__ void k_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags,
+                         double* box) {
+    unsigned qm = 0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
         const uint32_t i = order[k];
         if (i >= n) { flags[1] = 1; continue; }   // a sort that gave up leaves entries unwritten: any number
         pts[k] = make_dbl4(pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2], q[i]);
+        qm = max(qm, (unsigned)__double2hiint(q[i]) & 0x7FFFFFFFu);
     }
+    __shared__ unsigned block_max;
+    if (threadIdx.x == 0) block_max = 0;
+    __syncthreads();
+    qm = __reduce_max_sync(0xffffffffu, qm);
+    if ((threadIdx.x & 31) == 0) atomicMax(&block_max, qm);
+    __syncthreads();
+    unsigned* top = reinterpret_cast<unsigned*>(box + 5) + 1;
+    if (threadIdx.x == 0 && block_max > *(volatile unsigned*)top) atomicMax(top, block_max);
 }
 
 // One warp per cell: leaf points relative to the leaf centre, in FP32.
@@ -492,8 +505,8 @@ __global__ void k_check_tree(const int4* info, const int* lstart, int cap, long 
 }
 
 cudaError_t launch_gather(const double* pos, const double* q, const uint32_t* order, long long n, Dbl4* pts, int* flags,
-                          cudaStream_t s) {
-    k_gather<<<grid_for(n, 256, 4096), 256, 0, s>>>(pos, q, order, n, pts, flags);
+                          double* box, cudaStream_t s) {
+    k_gather<<<grid_for(n, 256, 4096), 256, 0, s>>>(pos, q, order, n, pts, flags, box);
     return cudaGetLastError();
 }
 
@@ -528,7 +541,7 @@ cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s) {
     // one block per SM, all resident (cooperative launch): the blocks wait for one another
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_levels), dim3(sms), dim3(kLvBlock), args, 0, s);
     if (e != cudaSuccess) return e;
-    if ((e = launch_gather(b.pos, b.q, b.order, n, b.pts, b.flags, s)) != cudaSuccess) return e;
+    if ((e = launch_gather(b.pos, b.q, b.order, n, b.pts, b.flags, b.box, s)) != cudaSuccess) return e;
     k_check_tree<<<grid_for(b.cap_cells, 256, 1216), 256, 0, s>>>(b.info, b.lstart, b.cap_cells, n, b.flags);
     return cudaGetLastError();
 }
