@@ -860,6 +860,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     const int fhigh = 32 * (int)P.maxspawn + 2 * kChunk;
     constexpr int kProbes = 16;  // victims probed in parallel per steal attempt (one lane each)
     bool token = false;          // warp-uniform: this warp holds its block's probe token
+    const bool host_reader = reads_host_word((uint32_t)wid, P.n_workers);
     // Tasks the warp takes for one step (warp-uniform): a k-clique kernel holds few of the tasks that
     // the warp serves, and whole batches of the others; so does its first claim, by the roots'
     // kind (claims of two made the lane-served counts slow: triangles of an R-MAT graph of scale 16
@@ -882,9 +883,8 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         const int cap = kAdaptive ? cap_now : 32;
         if ((iter & 63u) == 0u) {
             int ab = 0;
-            // the host's abort word is read by every 64th warp only, and not at the start: a
-            // mapped-memory read by each of thousands of warps delayed the first tasks
-            if (lane == 0) ab = abort_requested(P, (wid & 63) == 0 && (iter & 255u) == 64u) ? 1 : 0;
+            // (the host's word less often than the device's, and not at the start)
+            if (lane == 0) ab = abort_requested(P, host_reader && (iter & 255u) == 64u) ? 1 : 0;
             if (__shfl_sync(0xffffffffu, ab, 0)) break;
         }
         if constexpr (SCHED == SCHED_GLOBAL) {
@@ -1202,7 +1202,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                 } else if ((SCHED != SCHED_GLOBAL || (idle_n & 15u) == 1u) && ld_cg64(&P.ctl->roots_remaining.v) == 0ull) {
                     stop = 1;
                 } else if ((idle_n & 15u) == 1u) {
-                    if (abort_requested(P, (wid & 63) == 0 && (idle_n & 255u) == 17u)) stop = 1;
+                    if (abort_requested(P, host_reader && (idle_n & 255u) == 17u)) stop = 1;
                     else if (global_ns() > deadline) { raise_error(P, GTAP_ERR_TIMEOUT, -1, wid, P.timeout_ns); stop = 1; }
                 }
                 if (stop) *(volatile int*)&bidle->stop = 1;
@@ -1568,6 +1568,7 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
     int backoff = 32;
     int ftop = 0;
     const int fhigh = (int)P.maxspawn + 2 * kChunk;
+    const bool host_reader = reads_host_word((uint32_t)bid, P.n_workers);
 
     // per-phase clock accounting (thread 0): acquire, body, post-step, idle
     unsigned long long cy_acq = 0, cy_body = 0, cy_post = 0, cy_idle = 0;
@@ -1577,8 +1578,8 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
             uint32_t task = kNoTask;
             int state = 0;
             if (lane == 0) {
-                // (the host's abort word is read by every 64th block, and not at the start)
-                if ((iter & 15u) == 0u && abort_requested(P, (bid & 63) == 0 && (iter & 127u) == 64u)) {
+                // (the host's abort word less often than the device's, and not at the start)
+                if ((iter & 15u) == 0u && abort_requested(P, host_reader && (iter & 127u) == 64u)) {
                     state = 2;
                 } else if (bs.misc[1] != kNoTask) {
                     task = bs.misc[1];   // the task retained from the previous step
@@ -1693,7 +1694,7 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                     else if ((st_idle & 3ull) == 1ull && global_ns() > deadline) {
                         raise_error(P, GTAP_ERR_TIMEOUT, -1, bid, P.timeout_ns);
                         st = 2;
-                    } else if ((st_idle & 127ull) == 65ull && abort_requested(P, (bid & 63) == 0)) {
+                    } else if ((st_idle & 127ull) == 65ull && abort_requested(P, host_reader)) {
                         st = 2;
                     }
                 }

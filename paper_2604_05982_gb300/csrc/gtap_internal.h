@@ -239,6 +239,13 @@ struct KParams {
     uint64_t gq_mask;
 };
 
+// Whether a worker (warp or block) looks at the host's abort word.  The word is mapped host memory, whose
+// reads by thousands of warps delay the first tasks, so at most 127 do, spread evenly; but at
+// least 64, or all of a smaller grid, so that some of them are idle while others run long steps.
+GTAP_HD constexpr bool reads_host_word(uint32_t worker, uint32_t n_workers) {
+    return worker % (n_workers >= 64 ? n_workers / 64 : 1u) == 0;
+}
+
 // Debug-check failure codes (error detail = code << 32 | record id).
 enum DebugFault : unsigned long long {
     DBG_DOUBLE_ALLOC = 1, DBG_DOUBLE_FREE = 2, DBG_EXEC_NOT_ALLOCATED = 3, DBG_BAD_ID = 4,
