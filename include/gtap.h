@@ -86,7 +86,9 @@ typedef struct {
     int scheduler;          /* thread-mode queue management (GTAP_SCHED_*, default GTAP_SCHED_BATCHED);
                                the alternatives exist for the scheduler comparison of Sec. 6.5 */
     int idle_backoff_ns;    /* thread mode: longest sleep of an idle warp between steal rounds, 32..65536 ns
-                               (default 512); longer relieves L2 of idle probing, shorter spreads new work faster */
+                               (default 512); longer relieves L2 of idle probing, shorter spreads new work faster.
+                               One idle warp of a block probes at a time; the others wait for its turn in sleeps
+                               of up to 16 times this, at most 6400 ns or this value if it is longer */
 } gtap_config;
 
 /* Thread-mode scheduler designs compared in Sec. 6.5 ("GPU-Side Scheduler

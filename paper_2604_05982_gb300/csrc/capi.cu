@@ -722,6 +722,7 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
     P.seed = c->cfg.seed;
     P.steal_policy = c->cfg.steal_policy;
     P.idle_backoff_ns = c->cfg.idle_backoff_ns;
+    P.idle_wait_ns = idle_wait_bound(c->cfg.idle_backoff_ns);
     P.scratch = c->blocks;
     P.scratch_bytes = c->blocks_bytes;
     P.sq_seq = c->sq_seq;

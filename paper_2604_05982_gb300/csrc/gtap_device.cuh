@@ -793,19 +793,15 @@ struct BlockIdle {
 // Thread-mode scheduler loop (Algorithm 1), one instance per warp.
 // Dispatch is a functor: Dispatch::run(TaskCtx&) executes one step; program sets with
 // warp requests begin it, serve the requests by the whole warp, and finish it.
-// The longest sleep of an idle warp between steal rounds is a configuration
-// field (default 512 ns): longer sleeps relieve L2 of idle probing (the hashed
-// tree gained 8 % at 4 us) but slow the spread of work at start-up (fib and
-// N-Queens lost 15-25 % at 4 us), so the autotuner picks it per program.
-
+// The longest sleep of the probing warp between steal rounds is a configuration
+// field (default 512 ns): longer sleeps relieve L2 of idle probing, shorter ones
+// spread new work faster; the warps that wait for the token follow it
+// (idle_wait_bound).  The autotuner picks it per program.
 
 // Tasks a warp holds at a time when the whole warp serves them one after another
 // (Dispatch::kWarpRequests): 32 of them would keep one warp busy for
 // milliseconds while others find nothing to steal.
 constexpr int kWarpBatch = 2;
-
-// Longest sleep of an idle warp that waits for its block's probe token.
-constexpr int kIdleWaitMax = 6400;
 
 template <class Dispatch, int SCHED = SCHED_BATCHED>
 __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_warp) {
@@ -1038,7 +1034,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                 // up to 31 idle warps an SM: polling every 200 ns they took most of its issue
                 // slots from the one that works
                 __nanosleep(wait_ns);
-                wait_ns = min(wait_ns * 2, kIdleWaitMax);
+                wait_ns = min(wait_ns * 2, P.idle_wait_ns);
                 phase(kStIdleCy);
                 continue;
             }

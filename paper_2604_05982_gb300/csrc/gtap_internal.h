@@ -226,7 +226,7 @@ struct KParams {
     // serving mode (resident kernel)
     int serving;
     uint32_t inbox_cap, outbox_cap;
-    int pad1;
+    int idle_wait_ns;          // thread mode: longest sleep of an idle warp without its block's probe token
     InboxSlot* inbox;          // mapped pinned host memory (device pointers)
     OutboxEntry* outbox;
     HostFlags* hflags;
@@ -238,6 +238,12 @@ struct KParams {
     unsigned long long* gq;
     uint64_t gq_mask;
 };
+
+// Longest sleep of an idle warp that waits for its block's probe token, for a probing warp's longest
+// sleep b (gtap_config.idle_backoff_ns): a waiter reads shared memory only, so it may sleep 16 times as
+// long, but not beyond 6.4 us (the hashed tree ran 1.09 / 1.13 / 1.14 times as fast at 1.6 / 6.4 / 25.6 us
+// as at 0.2 us, but fib and N-Queens slower at 25.6), unless b itself is longer.
+GTAP_HD constexpr int idle_wait_bound(int b) { return b >= 6400 ? b : (b < 400 ? 16 * b : 6400); }
 
 // Whether a worker (warp or block) looks at the host's abort word.  The word is mapped host memory, whose
 // reads by thousands of warps delay the first tasks, so at most 127 do, spread evenly; but at
