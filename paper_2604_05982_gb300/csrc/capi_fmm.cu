@@ -149,7 +149,7 @@ struct gtap_fmm {
     gtap_fmm_config cfg{};
     int p = 6, nt = 84;
     bool mixed = false;
-    int sms = 0;
+    int sms = 0, refine_blocks = 0;
     cudaStream_t s = nullptr;
     HostTables ht;
     Tables tab{};
@@ -290,6 +290,7 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
         delete f;
         return GTAP_ERR_CUDA;
     }
+    f->refine_blocks = f->sms;
     f->ht.build(c.order);
     f->nt = f->ht.nt;
     const HostTables& h = f->ht;
@@ -329,7 +330,7 @@ gtap_status gtap_fmm_create(const gtap_fmm_config* cfg, gtap_fmm** out) {
     if (!f->counters.ensure(4 * sizeof(unsigned long long)) || !f->aux.ensure(sizeof(DttAux)) ||
         !f->box.ensure(8 * sizeof(double)) ||
         !f->bbox_part.ensure(6 * kBoxParts * sizeof(double)) || !f->lstart.ensure((kMaxLevel + 3) * sizeof(int)) ||
-        !f->block_sums.ensure(sizeof(int) * (size_t)f->sms) ||
+        !f->block_sums.ensure(sizeof(int) * (size_t)f->refine_blocks) ||
         !f->flags.ensure(4 * sizeof(int))) {
         delete f;
         return GTAP_ERR_NO_MEMORY;
@@ -368,6 +369,7 @@ gtap_status gtap_fmm_build(gtap_fmm* f, const double* pos, const double* q, int6
         b.vals[0] = f->vals0.as<uint32_t>();
         b.vals[1] = f->vals1.as<uint32_t>();
         b.work = f->work.p;
+        b.refine_blocks = f->refine_blocks;
         b.block_sums = f->block_sums.as<int>();
         b.geom = f->geom.as<Dbl4>();
         b.info = f->info.as<int4>();
@@ -552,6 +554,13 @@ gtap_status gtap_fmm_copy_lists(const gtap_fmm* f, int32_t* m2l, int32_t* p2p) {
             j.dst[2 * i + 1] = (int32_t)(tmp[i] & 0xFFFFFFFFull);
         }
     }
+    return GTAP_OK;
+}
+
+gtap_status gtap_debug_fmm_refine_blocks(gtap_fmm* f, int blocks) {
+    if (!f || blocks < 1 || blocks > (1 << 20)) return GTAP_ERR_INVALID_ARG;
+    if (!f->block_sums.ensure(sizeof(int) * (size_t)blocks)) return GTAP_ERR_NO_MEMORY;
+    f->refine_blocks = blocks;
     return GTAP_OK;
 }
 

@@ -129,7 +129,8 @@ struct TreeBufs {
     unsigned long long* keys[2];  // radix-sort ping-pong
     uint32_t* vals[2];
     void* work;                   // tree_work_bytes(n): counters, digit counts, look-back words
-    int* block_sums;              // [SM count]: children per block of the refinement
+    int refine_blocks;            // blocks of the refinement kernel (one per SM)
+    int* block_sums;              // [refine_blocks]: children per block of the refinement
     Dbl4* geom;
     int4* info;
     int4* lat;                    // cell centre on the level-21 lattice: (2i+1) << (21 - level) per axis, level
@@ -197,6 +198,8 @@ gtap_status dtt_env(const gtap_fmm* plan, int target, int source, DttEnv* out);
 }  // namespace fmm
 }  // namespace gtap
 
+// Test entry: later builds of the plan launch this many refinement blocks instead of one per SM.
+extern "C" gtap_status gtap_debug_fmm_refine_blocks(gtap_fmm* f, int blocks);
 // Test entry: the gather on device arrays (pts: n x 4, flags: 4 words), synchronised.
 extern "C" gtap_status gtap_debug_fmm_gather(const double* pos, const double* q, const uint32_t* order, int64_t n,
                                              double* pts, int32_t* flags);

@@ -9,8 +9,8 @@
 //   4. level-synchronous refinement: a cell of level l with more than
 //      leaf_size points (and l < 21) splits into its non-empty octants, found
 //      by search in the sorted codes; child cells are numbered breadth first by
-//      a scan of the per-cell child counts.  One cooperative kernel refines all
-//      levels, with a grid barrier between them;
+//      a scan of the per-cell child counts.  One kernel refines all levels, with
+//      a barrier of its running blocks between them;
 //   5. gather of the points into Morton order.
 // A build is 14 launches whatever the set (five per radix pass and five per
 // level made 85); most of a small set's build time was launches and the 7 x 20
@@ -255,8 +255,46 @@ __global__ void __launch_bounds__(kRsBlock) k_rs_pass(const unsigned long long* 
     }
 }
 
-// All blocks of a cooperative grid meet: `target` arrivals in all.  The wait is
-// bounded; a block that gives up marks the build as failed.
+// The state of the blocks that refine together, zeroed before the kernel.
+struct LvState {
+    unsigned started;   // blocks that have started
+    unsigned members;   // those that take part
+    unsigned met;       // their arrivals at barriers so far
+};
+constexpr int kLvGather = 1 << 10;   // looks at `started` (50 us) before the first block goes on with fewer
+
+// The blocks that refine together: all that start within about 50 us of the first.  They run, so they may
+// wait for one another, and a later block leaves.  (A cooperative launch waits until every block has
+// room: beside a served session that fills the chip but for a few blocks, until the session ends.)
+// Returns this block's number among them, or -1.
+__device__ __forceinline__ int join_members(LvState* st, int* members) {
+    __shared__ int rank_sh, members_sh;
+    if (threadIdx.x == 0) {
+        const unsigned r = atomicAdd(&st->started, 1u);
+        unsigned n = 0;
+        if (r == 0) {
+            volatile unsigned* started = &st->started;
+            for (int it = 0; it < kLvGather && *started < gridDim.x; ++it) __nanosleep(32);
+            n = *started;   // (a block that starts from here on has a number of at least n)
+            atomicExch(&st->members, n);
+        } else {
+            volatile unsigned* m = &st->members;
+            for (int it = 0; it < (1 << 22); ++it) {
+                n = *m;
+                if (n != 0) break;
+                __nanosleep(32);
+            }
+        }
+        rank_sh = r < n ? (int)r : -1;
+        members_sh = (int)n;
+    }
+    __syncthreads();
+    *members = members_sh;
+    return rank_sh;
+}
+
+// The members meet: `target` arrivals in all.  The wait is bounded; a block that
+// gives up marks the build as failed.
 __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, int* flags) {
     __shared__ int met;
     __syncthreads();
@@ -291,7 +329,7 @@ __device__ __forceinline__ int octant_bound(const unsigned long long* codes, int
     return a;
 }
 
-// Refinement of every level.  A block owns a contiguous range of the level's
+// Refinement of every level.  A member block owns a contiguous range of the level's
 // cells, 8 lanes to a cell (one per octant): first the octant boundaries and the
 // block's child count, then, after a barrier, the children from the prefix over
 // the blocks.
@@ -299,18 +337,22 @@ constexpr int kLvBlock = 256;
 
 __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* codes, int4* info, Dbl4* geom, int4* lat,
                                                      int* lstart, const double* box, int* bounds, int leaf, int cap,
-                                                     int* block_sums, unsigned* barrier, int* flags) {
+                                                     int* block_sums, LvState* state, int* flags) {
     __shared__ int red[kLvBlock / 32], total_sh, base_sh;
     const int t = threadIdx.x, lane = t & 31, o = t & 7, grp = t >> 3;
     const unsigned gshift = (unsigned)(lane & ~7);
     if (build_failed(flags)) return;
+    int members;
+    const int rank = join_members(state, &members);
+    if (rank < 0) return;
+    unsigned* barrier = &state->met;
     unsigned meet = 0;
     int l = 0;
     for (; l < kMaxLevel; ++l) {
         const int lo = __ldcg(lstart + l), hi = __ldcg(lstart + l + 1);
         if (lo == hi) break;
-        const int per = (hi - lo + (int)gridDim.x - 1) / (int)gridDim.x;
-        const int c0 = min(hi, lo + (int)blockIdx.x * per), c1 = min(hi, c0 + per);
+        const int per = (hi - lo + members - 1) / members;
+        const int c0 = min(hi, lo + rank * per), c1 = min(hi, c0 + per);
         const int shift = 3 * (20 - l);
         int mine = 0;   // children counted by this group (on its lane 0)
         for (int c = c0 + grp; c - grp < c1; c += kLvBlock / 8) {
@@ -337,15 +379,15 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
         if (t == 0) {
             int s = 0;
             for (int i = 0; i < kLvBlock / 32; ++i) s += red[i];
-            __stcg(block_sums + blockIdx.x, s);
+            __stcg(block_sums + rank, s);
         }
-        if (!grid_barrier(barrier, ++meet * gridDim.x, flags)) return;
+        if (!grid_barrier(barrier, ++meet * (unsigned)members, flags)) return;
         // children before this block's, and in all
         int before = 0, all = 0;
-        for (int i = t; i < (int)gridDim.x; i += kLvBlock) {
+        for (int i = t; i < members; i += kLvBlock) {
             const int v = __ldcg(block_sums + i);
             all += v;
-            if (i < (int)blockIdx.x) before += v;
+            if (i < rank) before += v;
         }
         before = (int)__reduce_add_sync(0xffffffffu, (unsigned)before);
         all = (int)__reduce_add_sync(0xffffffffu, (unsigned)all);
@@ -354,10 +396,10 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
         if (lane == 0) { atomicAdd(&total_sh, all); atomicAdd(&base_sh, before); }
         __syncthreads();
         if (total_sh > cap - hi) {   // the same decision in every block
-            if (blockIdx.x == 0 && t == 0) flags[0] = 1;
+            if (rank == 0 && t == 0) flags[0] = 1;
             return;
         }
-        if (blockIdx.x == 0 && t == 0) __stcg(lstart + l + 2, hi + total_sh);
+        if (rank == 0 && t == 0) __stcg(lstart + l + 2, hi + total_sh);
         const int cl = l + 1;
         const double cell = __ddiv_rn(box[3], (double)(1ull << cl));
         const double half = __dmul_rn(cell, 0.5);
@@ -406,10 +448,10 @@ __global__ void __launch_bounds__(kLvBlock) k_levels(const unsigned long long* c
                 __stcg(info + ch, make_int4(b0, b1 - b0, -1, cl << 8));
             }
         }
-        if (!grid_barrier(barrier, ++meet * gridDim.x, flags)) return;
+        if (!grid_barrier(barrier, ++meet * (unsigned)members, flags)) return;
     }
     // level l is empty (or past the deepest): the start entries after it equal its own
-    if (blockIdx.x == 0 && l < kMaxLevel) {
+    if (rank == 0 && l < kMaxLevel) {
         const int v = __ldcg(lstart + l);
         for (int k = l + 2 + t; k <= kMaxLevel + 1; k += kLvBlock) lstart[k] = v;
     }
@@ -514,7 +556,7 @@ cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s) {
     const long long n = b.n;
     cudaError_t e = cudaMemsetAsync(b.work, 0, tree_work_bytes(n), s);
     if (e != cudaSuccess) return e;
-    unsigned* counters = static_cast<unsigned*>(b.work);   // [0] box, [1] barrier, [8 + pass] tile tickets
+    unsigned* counters = static_cast<unsigned*>(b.work);   // [0] box, [4..6] LvState, [8 + pass] tile tickets
     unsigned* counts = reinterpret_cast<unsigned*>(static_cast<char*>(b.work) + kRsCounters);
     unsigned long long* look = reinterpret_cast<unsigned long long*>(static_cast<char*>(b.work) + kRsCounters + kRsCounts);
     k_bbox<<<grid_for(n, 256 * 4, kBoxParts), 256, 0, s>>>(b.pos, n, b.bbox_part, counters, b.box, b.geom, b.info, b.lat,
@@ -535,12 +577,10 @@ cudaError_t launch_tree(TreeBufs& b, int sms, cudaStream_t s) {
     b.codes = b.keys[cur];
     b.order = b.vals[cur];
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    unsigned* barrier = counters + 1;
-    void* args[] = {&b.codes, &b.info, &b.geom, &b.lat, &b.lstart, &b.box, &b.bounds, &b.leaf, &b.cap_cells,
-                    &b.block_sums, &barrier, &b.flags};
-    // one block per SM, all resident (cooperative launch): the blocks wait for one another
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_levels), dim3(sms), dim3(kLvBlock), args, 0, s);
-    if (e != cudaSuccess) return e;
+    k_levels<<<b.refine_blocks, kLvBlock, 0, s>>>(b.codes, b.info, b.geom, b.lat, b.lstart, b.box, b.bounds, b.leaf,
+                                                  b.cap_cells, b.block_sums, reinterpret_cast<LvState*>(counters + 4),
+                                                  b.flags);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_gather(b.pos, b.q, b.order, n, b.pts, b.flags, b.box, s)) != cudaSuccess) return e;
     k_check_tree<<<grid_for(b.cap_cells, 256, 1216), 256, 0, s>>>(b.info, b.lstart, b.cap_cells, n, b.flags);
     return cudaGetLastError();
