@@ -718,6 +718,7 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
     P.maxspawn = (uint32_t)maxspawn;
     P.stats = c->stats;
     P.host_abort = c->host_abort_dev;
+    P.host_word_mask = host_word_mask(P.n_workers);
     P.timeout_ns = c->cfg.timeout_ns;
     P.seed = c->cfg.seed;
     P.steal_policy = c->cfg.steal_policy;

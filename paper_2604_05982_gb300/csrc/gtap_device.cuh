@@ -856,7 +856,6 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     const int fhigh = 32 * (int)P.maxspawn + 2 * kChunk;
     constexpr int kProbes = 16;  // victims probed in parallel per steal attempt (one lane each)
     bool token = false;          // warp-uniform: this warp holds its block's probe token
-    const bool host_reader = reads_host_word((uint32_t)wid, P.n_workers);
     // Tasks the warp takes for one step (warp-uniform): a k-clique kernel holds few of the tasks that
     // the warp serves, and whole batches of the others; so does its first claim, by the roots'
     // kind (claims of two made the lane-served counts slow: triangles of an R-MAT graph of scale 16
@@ -880,7 +879,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         if ((iter & 63u) == 0u) {
             int ab = 0;
             // (the host's word less often than the device's, and not at the start)
-            if (lane == 0) ab = abort_requested(P, host_reader && (iter & 255u) == 64u) ? 1 : 0;
+            if (lane == 0) ab = abort_requested(P, ((uint32_t)wid & P.host_word_mask) == 0 && (iter & 255u) == 64u) ? 1 : 0;
             if (__shfl_sync(0xffffffffu, ab, 0)) break;
         }
         if constexpr (SCHED == SCHED_GLOBAL) {
@@ -958,6 +957,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                     count(kStPopped, claim);
                 }
                 __syncwarp();
+                if (cnt == 0) continue;   // (a claim that lost every race: the queue is not known to be empty)
             }
         } else {
             // ---- PopBatch (Algorithm 2) from the own queue: the retained class, else the fullest (DAQ).
@@ -1006,6 +1006,11 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                         count(kStPopped, claim);
                     } else {
                         __syncwarp();
+                        // The fullest class was stolen (its hint is now 0): the other own classes come before
+                        // any idling.  So a warp that takes the probe token has no class left to pop, and
+                        // only its own pushes raise a hint: none works with the token that the block's
+                        // others wait for.
+                        if (cnt == 0) continue;
                     }
                 }
             }
@@ -1013,21 +1018,14 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
         phase(kStPop);
         // ---- Idle: wait for the block's probe token (not with the central queue, which has no victims).
         if (SCHED != SCHED_GLOBAL && cnt == 0 && !token) {
-            // The fullest class may have been stolen (its hint is now 0): the other own classes come
-            // first.  A warp that takes the token has no class left to pop, and only its own pushes
-            // raise a hint, so no warp works with the token that the block's others wait for.
             int got = 0;
             if (lane == 0) {
                 volatile BlockIdle* b = bidle;
-                int left = 0;
-                for (int k = 0; k < Q; ++k) left |= ws.hint[k];   // (never negative)
                 if (b->stop) got = 2;
-                else if (left != 0) got = 3;
                 else if (b->token == 0 && atomicCAS_block(&bidle->token, 0, 1) == 0) got = 1;
             }
             got = __shfl_sync(0xffffffffu, got, 0);
             if (got == 2) break;
-            if (got == 3) continue;
             token = got == 1;
             if (!token) {
                 ++idle_n;
@@ -1198,7 +1196,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
                 } else if ((SCHED != SCHED_GLOBAL || (idle_n & 15u) == 1u) && ld_cg64(&P.ctl->roots_remaining.v) == 0ull) {
                     stop = 1;
                 } else if ((idle_n & 15u) == 1u) {
-                    if (abort_requested(P, host_reader && (idle_n & 255u) == 17u)) stop = 1;
+                    if (abort_requested(P, ((uint32_t)wid & P.host_word_mask) == 0 && (idle_n & 255u) == 17u)) stop = 1;
                     else if (global_ns() > deadline) { raise_error(P, GTAP_ERR_TIMEOUT, -1, wid, P.timeout_ns); stop = 1; }
                 }
                 if (stop) *(volatile int*)&bidle->stop = 1;
@@ -1564,7 +1562,6 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
     int backoff = 32;
     int ftop = 0;
     const int fhigh = (int)P.maxspawn + 2 * kChunk;
-    const bool host_reader = reads_host_word((uint32_t)bid, P.n_workers);
 
     // per-phase clock accounting (thread 0): acquire, body, post-step, idle
     unsigned long long cy_acq = 0, cy_body = 0, cy_post = 0, cy_idle = 0;
@@ -1575,7 +1572,7 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
             int state = 0;
             if (lane == 0) {
                 // (the host's abort word less often than the device's, and not at the start)
-                if ((iter & 15u) == 0u && abort_requested(P, host_reader && (iter & 127u) == 64u)) {
+                if ((iter & 15u) == 0u && abort_requested(P, ((uint32_t)bid & P.host_word_mask) == 0 && (iter & 127u) == 64u)) {
                     state = 2;
                 } else if (bs.misc[1] != kNoTask) {
                     task = bs.misc[1];   // the task retained from the previous step
@@ -1690,7 +1687,7 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                     else if ((st_idle & 3ull) == 1ull && global_ns() > deadline) {
                         raise_error(P, GTAP_ERR_TIMEOUT, -1, bid, P.timeout_ns);
                         st = 2;
-                    } else if ((st_idle & 127ull) == 65ull && abort_requested(P, host_reader)) {
+                    } else if ((st_idle & 127ull) == 65ull && abort_requested(P, ((uint32_t)bid & P.host_word_mask) == 0)) {
                         st = 2;
                     }
                 }

@@ -210,6 +210,7 @@ struct KParams {
     uint32_t warp_smem;       // thread mode: shared bytes per warp (runtime part + the program set's warp area)
     WorkerStats* stats;
     volatile int* host_abort; // mapped pinned host word, may be null
+    uint32_t host_word_mask;  // workers whose number has none of these bits read it
     uint64_t timeout_ns;
     uint64_t seed;
     int steal_policy;
@@ -246,10 +247,17 @@ struct KParams {
 GTAP_HD constexpr int idle_wait_bound(int b) { return b >= 6400 ? b : (b < 400 ? 16 * b : 6400); }
 
 // Whether a worker (warp or block) looks at the host's abort word.  The word is mapped host memory, whose
-// reads by thousands of warps delay the first tasks, so at most 127 do, spread evenly; but at
+// reads by thousands of warps delay the first tasks, so at most 128 do, spread evenly; but at
 // least 64, or all of a smaller grid, so that some of them are idle while others run long steps.
+// The mask of the worker number is a kernel parameter (a quotient kept in a register of the loop slowed the
+// kernel with every program by 2 %).
+GTAP_HD constexpr uint32_t host_word_mask(uint32_t n_workers) {
+    uint32_t m = 1;
+    while (2 * m * 64 <= n_workers) m *= 2;
+    return m - 1;
+}
 GTAP_HD constexpr bool reads_host_word(uint32_t worker, uint32_t n_workers) {
-    return worker % (n_workers >= 64 ? n_workers / 64 : 1u) == 0;
+    return (worker & host_word_mask(n_workers)) == 0;
 }
 
 // Debug-check failure codes (error detail = code << 32 | record id).
