@@ -666,12 +666,12 @@ static gtap_status plan_and_enqueue(gtap_ctx* c, cudaStream_t s, LaunchPlan* lp,
         pset = thread_kernel_pset(c->registered);
         maxspawn = thread_kernel_maxspawn(pset);
         frame_bytes = c->cfg.frame_bytes ? (uint32_t)c->cfg.frame_bytes : thread_record_bytes(pset);
-        P.warp_roots = serving ? 1 : 0;
+        P.warp_roots = serving ? kWarpRootsServing : 0;
         for (const RootDesc& d : c->pending_roots)
             if (d.type == T_KCLIQUE_ROOT) {
                 gtap_kclique_args a;
                 std::memcpy(&a, d.env, sizeof(a));
-                if (a.algorithm != GTAP_KCLIQUE_PIVOT && a.k > 3) P.warp_roots = 1;
+                if (!serving && a.algorithm != GTAP_KCLIQUE_PIVOT && a.k > 3) P.warp_roots = kWarpRootsBatch;
             }
         // the programs' warp area (80 KB an SM) is for warp requests; without them it is left to the L1
         // cache (triangles of an R-MAT graph of scale 16: 1.32 -> 0.96 ms; 6-cliques by pivoting,

@@ -189,6 +189,8 @@ enum StatWord : int {
 };
 static_assert(sizeof(WorkerStats) == kStatWords * 8, "StatWord names the words of WorkerStats");
 
+constexpr int kWarpRootsBatch = 1, kWarpRootsServing = 2;
+
 // Kernel parameters (passed by value).
 struct KParams {
     char* frames;
@@ -215,7 +217,8 @@ struct KParams {
     uint64_t seed;
     int steal_policy;
     int idle_backoff_ns;      // thread mode: longest sleep of an idle warp between steal rounds
-    int warp_roots;           // some root's tasks may be served by the whole warp (k-clique by orientation, k > 3)
+    int warp_roots;           // some root's tasks may be served by the whole warp (k-clique by orientation, k > 3):
+                              // kWarpRootsBatch, or in a served session, where any may come, kWarpRootsServing
     char* scratch;            // scratch blocks for programs (k-clique candidate sets), kScratchBlock bytes each
     uint64_t scratch_bytes;   // bytes of the block region
     unsigned long long* sq_seq;   // free-block queue: sequence numbers and block ids

@@ -1071,7 +1071,9 @@ __device__ __forceinline__ bool kc_warp_root(const gtap_kclique_args& e) {
 static __device__ bool kclique_range_begin(TaskCtx& c, KcReq& q) {
     const KcRangeSpawn a = c.load<KcRangeSpawn>();
     const gtap_kclique_args& e = kc_env(c.P, a.root);
-    q.warp_task = kc_warp_root(e);
+    // (beside roots whose tasks ask the warp, a triangle count's are held few at a time as well: a claim of
+    // 32 would take theirs too; 3-, 4- and 5-cliques of one R-MAT graph of scale 13 in one run 2.8 against 4.8 ms)
+    q.warp_task = kc_warp_root(e) || (e.algorithm != GTAP_KCLIQUE_PIVOT && c.P.warp_roots == kWarpRootsBatch);
     if (c.pc() != 0) { c.ret(a.acc + a.local); return false; }
     const uint32_t n = a.hi - a.lo;
     if (n > (uint32_t)kKcFan) {

@@ -32,3 +32,15 @@ def test_branches_of_sets_beyond_the_warp_buffer_fill_the_warp():
     r = runner.kclique(g, 4, n_queues=4, route=1, ranges=[(0, 100)], grid_blocks=8)
     assert r.values == [sum((n - 1 - w) * (n - 2 - w) // 2 for w in range(1, 101))]
     assert r.stats["tasks_executed"] > 8 * r.stats["steps"]
+
+
+def test_triangle_tasks_beside_tasks_for_the_warp_are_held_few_at_a_time():
+    # a full batch claimed for triangles could hold 4-clique tasks, which the warp serves one by one
+    n, e = inputs.rmat_graph(12, 16, seed=5)
+    g = runner.DeviceGraph(n, e)
+    with runner.Context(G.GTAP_MODE_THREAD, 4, scratch_bytes=1 << 30) as c:
+        t = c.register("kclique")
+        handles = [c.spawn(t, g.args(k, 64, 1)) for k in (3, 4)]
+        c.run()
+        assert [c.result_u64(h) for h in handles] == [oracle.kclique(n, e, k) for k in (3, 4)]
+        assert c.stats()["tasks_executed"] <= 2 * c.stats()["steps"]
