@@ -1338,23 +1338,6 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
             }
             int kept = 0;
             int gbad = 0;
-            // One queue: the first staged tasks are kept, the others go to the ring in order, with no
-            // classes to rank.
-            if (Dispatch::kOneQueuePath && SCHED != SCHED_GLOBAL && Q == 1) {
-                for (int i = lane; i < nst; i += 32) {
-                    const uint32_t id = ws.staged_id[i];
-                    if (i < nkeep) {
-                        ws.retained[i] = id;
-                        dbg_log(P, id, 9, wid, iter, (unsigned)i);
-                    } else {
-                        const uint32_t pos = ws.tail[0] + (uint32_t)(i - nkeep);
-                        __stcg(&myring[pos & cap_mask], id);
-                        dbg_log(P, id, 6, wid, iter, pos & 0xFFFF);
-                    }
-                }
-                if (lane == 0) ws.push_off[0] = nst - nkeep;
-                __syncwarp();
-            } else
             for (int base = 0; base < nst; base += 32) {
                 const int i = base + lane;
                 const bool valid = i < nst;

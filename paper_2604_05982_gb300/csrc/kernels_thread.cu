@@ -10,11 +10,6 @@ namespace gtap {
 
 template <unsigned PSET>
 struct ThreadDispatch {
-    // Tasks of a single queue are retained and pushed without ranking classes: the hashed tree's
-    // dependent steps gain (4.89 -> 4.66 ms for 2000 root children); compiled into the other kernels
-    // it gained nothing (fib) or made the loop slower (N-Queens 998 -> 1026 us, the kernel with
-    // every program 65 -> 69 ms on the served mix).
-    static constexpr bool kOneQueuePath = PSET == PS_UTS;
     // A step may leave a request that the whole warp serves before the lane finishes the step.
     static constexpr bool kWarpRequests = (PSET & PS_KCLIQUE) != 0;
     static constexpr bool kAdaptiveBatch = PSET == PS_KCLIQUE;   // the batch follows the tasks (kWarpBatch or 32)
