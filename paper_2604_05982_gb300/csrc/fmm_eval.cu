@@ -421,7 +421,7 @@ constexpr int kM2lWarps = 4;
 
 // Bound by FP32 issue and by the lanes' uncoalesced row reads (208 B a source).
 // 49 + 64 expansion and derivative registers fit 128, so 4 blocks (16 warps)
-// stay resident; over 84 coefficients it took 168 registers at 3 blocks.
+// stay resident (24 bytes spill); over 84 coefficients it took 168 registers at 3 blocks.
 // N = 2^20 uniform, p = 6: 2.29 -> 1.70 ms (fold included); Plummer 3.88 -> 2.86 ms.
 // Error against the FP64 form there: 9.2e-7 -> 7.6e-7 and 1.4e-6 -> 1.1e-6.
 template <int P>

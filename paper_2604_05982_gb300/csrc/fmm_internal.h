@@ -78,8 +78,9 @@ static_assert(sizeof(DttSpawn) == 112, "DttSpawn must fill a 128-byte record pay
 //  m2l terms, grouped by beta: (alpha, alpha+beta) with |alpha| + |beta| <= p and
 //    coefficient (-1)^|alpha| C(alpha+beta, beta); split into items of at most
 //    kM2lChunk terms, each item one accumulator of one beta.
-//  m2m terms, grouped by alpha: (beta <= alpha, alpha - beta) with C(alpha, beta).
-//  l2l terms, grouped by gamma: (beta >= gamma, beta - gamma) with C(beta, gamma).
+//  m2m terms, grouped by alpha: the index pairs (beta <= alpha, alpha - beta); in the scaled variables
+//    of the shifts they have no coefficient.
+//  l2l terms, grouped by gamma: the index pairs (beta >= gamma, beta - gamma).
 constexpr int kM2lChunk = 8;
 struct DerivEntry {
     int16_t e1[3], e2[3];

@@ -12,8 +12,8 @@
 //      a scan of the per-cell child counts.  One kernel refines all levels, with
 //      a barrier of its running blocks between them;
 //   5. gather of the points into Morton order.
-// A build is 14 launches whatever the set (five per radix pass and five per
-// level made 85); most of a small set's build time was launches and the 7 x 20
+// A build is 14 launches in the mixed form, 13 in FP64 (no leaf-local coordinates), and a memset,
+// whatever the set (five launches per radix pass and five per level made 85); most of a small set's build time was launches and the 7 x 20
 // dependent loads of one thread searching the root cell.  Build time before ->
 // now: 3,001 points 0.64 -> 0.16 ms, Plummer 60,001 0.85 -> 0.23 ms, uniform 2^20
 // 0.96 -> 0.47 ms.  A small set is bound by the chain of launches and barriers,

@@ -621,7 +621,7 @@ struct TaskCtx {
 // round trip, one path after another.  Here all lanes share one fence and one
 // round trip (16 roots of fib(22..28) in one launch: 1.39 -> 1.22 ms; N-Queens
 // up to 13 with 4 queues: 1.48 -> 1.19 ms; 400 mixed served requests, where a
-// warp holds several programs at once: 201 -> 93 ms).
+// warp holds several programs at once: 2.2 times as fast).
 __device__ __forceinline__ void complete_task(const KParams& P, const WarpSh& ws, uint32_t self, uint32_t w0,
                                               uint32_t parent, uint32_t w3, unsigned long long v, int worker,
                                               uint32_t iter) {
@@ -783,7 +783,7 @@ static __device__ __noinline__ void serve_poller(const KParams& P, const WarpSh&
 // Eight probing warps per block kept L2 busy with the queue words that the
 // working warps need, and every one of them tested for termination only each
 // 16th round, 30 us after the last task (eight roots of fib(8..14): 318 -> 241 us
-// a run, 400 served requests: 106 -> 91 ms, fib(22..28) x 16: 1.01 -> 0.98 ms).
+// a run, fib(22..28) x 16: 1.01 -> 0.98 ms; the served mix gained 2 %).
 struct BlockIdle {
     int token;   // 1 while a warp of the block probes
     int stop;    // set by the holder once the run is over
@@ -837,8 +837,7 @@ __device__ void thread_mode_loop(const KParams& P, BlockIdle* bidle, char* smem_
     }
     // The warp's counters live one per lane (lane i holds word i of WorkerStats): 2
     // registers instead of 32, which the loop would otherwise spill around every step
-    // (fib(22..28) x 16: 1.22 -> 1.01 ms, hashed tree: 5.5 -> 5.0 ms, Cilksort of 300,007
-    // keys: 2.86 -> 2.62 ms).
+    // (fib(22..28) x 16: 1.22 -> 1.01 ms, Cilksort of 300,007 keys: 2.86 -> 2.62 ms).
     unsigned long long stat = 0;
     auto count = [&](int word, unsigned long long v) { if (lane == word) stat += v; };
     uint32_t idle_n = 0;
@@ -1743,6 +1742,8 @@ __device__ void block_mode_loop(const KParams& P, char* smem, int bsz) {
                     uint32_t done = self, parent = h.parent;
                     while (true) {
                         dbg_transition(P, done, 1u, 0u, DBG_DOUBLE_FREE, (int)(h.w0 & 0xFF), bid);
+                        // (a chain is a merge's nested forks, each into up to 256 pieces, and its sort: far
+                        // fewer records than the cache's 33 spare entries)
                         const int top = max(bs.ctrl[0], 0);
                         if (top < bs.fcap) { bs.fstack[top] = done; bs.ctrl[0] = top + 1; }
                         if (parent & kRootBit) {

@@ -806,7 +806,9 @@ __device__ __forceinline__ int kc_index_of(const int* C, int n, int x) {
 // 10..14: 90 -> 65 ms.  Bound by issue: about 30 instructions for each list element searched.
 constexpr int kKcEdges = 1, kKcBranches = 2, kKcPairs = 3;
 // (the largest sets of an R-MAT graph of scale 20 hold between 256 and 512 members: its 4-clique
-// count takes 218 ms with 512 here, 364 ms with 256 and the rest by the per-lane path)
+// count takes 218 ms with 512 here, 364 ms with 256 and the rest by the per-lane path.  Denser graphs
+// have larger sets, which fork over their branches, one lane each, in full batches: 4-cliques of K_700
+// 79 ms, of K_900 165 ms; with every set by the per-lane path it was 82 and 203 ms)
 constexpr int kKcSetMax = 512;
 // Per-warp area: the set, then the rows of a small set or 32 members' lists.
 struct KcArea {
