@@ -463,7 +463,11 @@ gtap_status gtap_autotune(int mode, const char* program, const void* root_args, 
 #define GTAP_FMM_FP64 0   /* every kernel in FP64 */
 #define GTAP_FMM_MIXED 1  /* P2M, M2L, L2P, P2P and the deeper M2M/L2L in FP32, the M2L and
                              P2P sums compensated (Kahan); M2M/L2L into cells of the top
-                             fp64_levels levels in FP64.  Expansions are stored in FP64. */
+                             fp64_levels levels in FP64.  Expansions are stored in FP64.
+                             FP32 powers of the distances bound the point set's extent: 1e-3 to
+                             1e5 at every order (1e-4 to 1e7 at order 6, 1e-8 to 1e10 at order 3);
+                             scale other sets, or use FP64.  Points of one leaf whose FP32
+                             coordinates about its centre are equal do not interact. */
 
 typedef struct {
     int order;             /* expansion order p, 1..8 (default 6) */
